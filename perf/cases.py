@@ -65,7 +65,7 @@ def draw(rng):
                     precision=rng.choice([0, 1, 1]))
     if kind == "tessellate":
         return dict(kind=kind, n=side(500, 2_000_000), bx=1.0, by=rng.uniform(0.5, 2.0), bz=rng.uniform(0.5, 2.0))
-    recipe = rng.choice(["wave", "tube", "blast", "shear", "gresho"])
+    recipe = rng.choice(["wave", "tube", "shear", "gresho"] + ["blast"] * (kind != "host"))
     s = side(8, 32 if kind == "stages" else (110 if kind == "host" else 200))
     if recipe == "tube":
         nx, ny, nz = 4 * s, max(4, s // 2), max(4, s // 2 - 1)
@@ -253,6 +253,8 @@ def prepare(case, seed):
     U = ctx.mm_prims_to_charges(mesh, rho, vel, pres)
     _deposit(case, pos, U)
     st.update(ctx=ctx, box=box, pos=pos, U=U, dt=torch.empty(1, dtype=F8, device=dev))
+    if case["kind"] == "step":
+        st.update(pos0=pos.clone(), U0=U.clone())
     if case["kind"] == "host":
         st["pos"] = pos.cpu().pin_memory()
         st["U"] = U.cpu().pin_memory()
@@ -284,6 +286,7 @@ def _prepare_batch(case, gen, dev, st):
         U[:, sl] = helper.mm_prims_to_charges(mesh, rho, vel[:, sl].contiguous(), torch.ones_like(rho))
     helper.close()
     torch.cuda.synchronize()
+    st.update(pos0=pos.clone(), U0=U.clone())
     st.update(ctx=binding.Context(stream=stream, **_config(case, 5.0 / 3.0)), stream=stream, pos=pos, U=U, off=off,
               boxes=np.ones((len(sizes), 3)), dt=torch.empty(len(sizes), dtype=F8, device=dev))
     return st
@@ -291,6 +294,11 @@ def _prepare_batch(case, gen, dev, st):
 
 def run(st):
     ctx, kind = st["ctx"], st["kind"]
+    if kind in ("step", "batch"):
+        # each pass is the same step: from the snapshot the program keeps, not
+        # hundreds of steps into a run (an unregularised blast mesh tangles there)
+        st["pos"].copy_(st["pos0"])
+        st["U"].copy_(st["U0"])
     if kind == "step":
         ctx.mm_step(st["pos"], st["U"], st["box"], dt_out=st["dt"])
     elif kind == "batch":
