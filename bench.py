@@ -190,14 +190,12 @@ def clip_roofline(direct, filtered, ms, n, clip_filter):
     return out
 
 
-# DRAM traffic of one k_clip launch, from an ncu capture of one launch on the
-# 128^3 shear layer (dram__bytes_read.sum + dram__bytes_write.sum = 459,768,320
-# + 1,439,416,576 bytes over 2,097,152 cells; filtered clipping, two warps per
-# block), per cell; it scales with the cells of the launch.  Valid only for the
-# clipper source it was taken on: the digest of the clipping kernel's sources
-# must match, else the figure is withheld.
-CLIP_TRAFFIC = {"sources": ("csrc/mm_clip.cu", "csrc/mm_internal.cuh"), "sha256_16": "ed02d4137c2d00bd",
-                "bytes_per_cell": 1908677632 / 2097152, "cells_captured": 2097152}
+# DRAM traffic of the clipping kernels per cell, from an ncu capture of one
+# tessellation's launches.  Valid only for the clipper sources it was taken on:
+# the digest of the clipping kernels' sources must match, else the figure is
+# withheld.  (None: no capture of the current kernels.)
+CLIP_TRAFFIC = {"sources": ("csrc/mm_cells.cu", "csrc/mm_clip.cu", "csrc/mm_clip.cuh", "csrc/mm_internal.cuh"),
+                "sha256_16": "", "bytes_per_cell": None, "cells_captured": 2097152}
 
 
 def clip_sources_digest():
@@ -210,7 +208,7 @@ def clip_sources_digest():
 
 
 def clip_traffic(n, clip_filter):
-    """DRAM bytes of one k_clip launch on n cells, scaled from the 128^3
+    """DRAM bytes of the clipping launches on n cells, scaled from the 128^3
     capture by cell count; None when the capture does not cover the current
     clipper source or clipper variant."""
     if not clip_filter or CLIP_TRAFFIC["bytes_per_cell"] is None:
@@ -827,7 +825,7 @@ def run_ours(args, world, rank, local):
         roofline = clip_roofline(tdirect, tstats, dom_ms, n, args.clip_filter)
         roofline["traffic"] = clip_traffic(n, args.clip_filter)
         if roofline["traffic"] is not None:
-            roofline["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_clip launch "
+            roofline["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the clipping launches "
                                           "at 128^3, scaled by cells")
     else:
         byts = algorithmic_bytes(dom, n, nf)

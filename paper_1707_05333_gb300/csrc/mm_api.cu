@@ -482,10 +482,21 @@ static mm_status tess_enqueue(mm_ctx *c, const double *pos, bool fixed)
     Slots sl = slots();
     const int prec = c->cfg.clip_filter ? 1 : 0;
     stage_mark(c, MM_STAGE_CLIP, true);
+    // The filtered clipper takes all cells eight lanes each and leaves the
+    // unusual ones to the warp-per-cell clipper (the list shares its storage
+    // with the face counts written later).  The work counters are those of the
+    // warp-per-cell clipper.
+    int *list = nullptr;
+    if (prec == 1 && !c->cfg.collect_stats && n >= CELLS_MIN) {
+        list = P<int>(c->emit_cnt);
+        launch_cells(P<double4_32a>(c->sorted), P<float4>(c->sortedf), P<int>(c->bin_start), n, boxes, cbox,
+                     c->cfg.cand_cap, P<double>(c->vol), P<double>(c->cen), sl, list, &c->st->nlist, s);
+        c->launches += 2;
+    }
     launch_clip(P<double4_32a>(c->sorted), P<float4>(c->sortedf), P<int>(c->bin_start), n, boxes, cbox, prec,
                 c->cfg.collect_stats,
                 c->cfg.clip_warps, c->cfg.cand_cap, c->cfg.clip_sort, P<double>(c->vol), P<double>(c->cen), sl, c->st,
-                s);
+                list, &c->st->nlist, s);
     // cells over a capacity of the main clipper, again with the large one
     // (one warp per overflow row; nothing to do when no cell overflowed)
     launch_clip_big(P<double4_32a>(c->sorted), P<float4>(c->sortedf), P<int>(c->bin_start), n, boxes, cbox, prec,

@@ -36,11 +36,10 @@
 // plane's offset, so vertices on it (co-spherical generators of exact
 // lattices, where one point has several representations with different
 // rounding) are kept consistently.
-#include "mm_internal.cuh"
+#include "mm_clip.cuh"
 
 namespace mm {
 
-constexpr unsigned FULL = 0xffffffffu;
 #ifndef MM_CLIP_MAXNREG
 #define MM_CLIP_MAXNREG 128  // registers per thread of the clipping kernel
 #endif
@@ -139,19 +138,6 @@ struct PMask<128> {
     __device__ __forceinline__ bool operator!=(const PMask &o) const { return w != o.w || h != o.h; }
 };
 
-// Rarely taken integer work of the gather, kept out of line so that the hot
-// loop around it stays small (the kernel is sensitive to instruction-cache
-// misses): floor(a / b) for b > 0 (images beyond the neighbouring boxes), and
-// the bin offsets of entry t of ring block rh of side nb = 2 rh + 1 (rings 3
-// and beyond).
-__device__ __noinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
-__device__ __noinline__ int3 ring_offset(int t, int nb, int rh)
-{
-    return make_int3(t % nb - rh, (t / nb) % nb - rh, t / (nb * nb) - rh);
-}
-
-__device__ __forceinline__ unsigned lanemask_lt() { return (1u << (threadIdx.x & 31)) - 1u; }
-
 // Warp-wide sums of four values, on every lane, in a fixed order.  Each
 // exchange halves the number of partial sums a lane keeps (lanes with bit 4
 // clear keep a and b, the others c and d; then bit 3 splits those), so a
@@ -187,12 +173,6 @@ __device__ __forceinline__ long long dbits_of_float(float f)
     return __double_as_longlong((double)f);
 }
 
-// Magnitude order of doubles by their bit patterns (non-negative values, or
-// absolute values): an integer comparison in place of an FP64 one.
-__device__ __forceinline__ long long abs_bits(double x)
-{
-    return __double_as_longlong(x) & 0x7fffffffffffffffLL;
-}
 // Warp-wide maximum of a non-negative 64-bit value: the high words first,
 // then the low words of the lanes holding the largest high word.
 __device__ __forceinline__ long long warp_max_nonneg(long long v)
@@ -233,83 +213,6 @@ __device__ __forceinline__ int first_free(const PMask<128> &live, int np)
     const unsigned long long f0 = u0 & ~live.w, f1 = u1 & ~live.h;
     if (f0) return __ffsll((long long)f0) - 1;
     return f1 ? 64 + __ffsll((long long)f1) - 1 : -1;
-}
-
-// Intersection of planes a, b, c in FP64 with explicitly rounded operations
-// (so every caller gets the same bits):
-// x = (o_a (q_b x q_c) + o_b (q_c x q_a) + o_c (q_a x q_b)) / det(q_a, q_b, q_c).
-template <class S_t>
-__device__ __forceinline__ void vertex64(const S_t &S, int a, int b, int c, double &x, double &y, double &z)
-{
-    const double ax = S.px[a], ay = S.py[a], az = S.pz[a], ao = S.po[a];
-    const double bx = S.px[b], by = S.py[b], bz = S.pz[b], bo = S.po[b];
-    const double cx = S.px[c], cy = S.py[c], cz = S.pz[c], co = S.po[c];
-    const double bcx = __fma_rn(by, cz, -__dmul_rn(bz, cy)), bcy = __fma_rn(bz, cx, -__dmul_rn(bx, cz)),
-                 bcz = __fma_rn(bx, cy, -__dmul_rn(by, cx));
-    const double cax = __fma_rn(cy, az, -__dmul_rn(cz, ay)), cay = __fma_rn(cz, ax, -__dmul_rn(cx, az)),
-                 caz = __fma_rn(cx, ay, -__dmul_rn(cy, ax));
-    const double abx = __fma_rn(ay, bz, -__dmul_rn(az, by)), aby = __fma_rn(az, bx, -__dmul_rn(ax, bz)),
-                 abz = __fma_rn(ax, by, -__dmul_rn(ay, bx));
-    const double det = __fma_rn(ax, bcx, __fma_rn(ay, bcy, __dmul_rn(az, bcz)));
-    const double inv = __drcp_rn(det);
-    x = __dmul_rn(__fma_rn(ao, bcx, __fma_rn(bo, cax, __dmul_rn(co, abx))), inv);
-    y = __dmul_rn(__fma_rn(ao, bcy, __fma_rn(bo, cay, __dmul_rn(co, aby))), inv);
-    z = __dmul_rn(__fma_rn(ao, bcz, __fma_rn(bo, caz, __dmul_rn(co, abz))), inv);
-}
-
-// The exact-path predicate: is vertex v strictly beyond the plane x.q <= off?
-__device__ __forceinline__ bool beyond64(double qx, double qy, double qz, double off, double x, double y, double z)
-{
-    return __fma_rn(qx, x, __fma_rn(qy, y, __dmul_rn(qz, z))) > off;
-}
-
-// |q|^2 / 2 from the bit pattern of |q|^2: halving a normal double lowers its
-// exponent by one, an integer operation.
-__device__ __forceinline__ double half_of(long long d2bits)
-{
-    if (((d2bits >> 52) & 0x7ff) > 1) return __longlong_as_double(d2bits - (1LL << 52));
-    return 0.5 * __longlong_as_double(d2bits);
-}
-
-__device__ __forceinline__ long long r2_bits64(double x, double y, double z)
-{
-    return __double_as_longlong(__fma_rn(x, x, __fma_rn(y, y, __dmul_rn(z, z))));
-}
-
-// Intersection of planes a, b, c in FP32 with a bound on its distance to the
-// exact intersection.  With P = |q_a||q_b||q_c|, H = P / |det| >= 1 and
-// u = 2^-24, first-order rounding analysis of Cramer's rule (inputs rounded
-// to FP32, cross products, determinant, numerator, scaling) gives
-// |v~ - v| <= u H (5.5 sum|q| + 13 |v|); the bound used is three times that.
-// Ill-conditioned intersections get an infinite bound (always checked in FP64).
-template <class S_t>
-__device__ __forceinline__ void vertex32(const S_t &S, int a, int b, int c, float &x, float &y, float &z,
-                                         float &err)
-{
-    const float4 Pa = S.pf[a], Pb = S.pf[b], Pc = S.pf[c];
-    const float ax = Pa.x, ay = Pa.y, az = Pa.z, ao = Pa.w;
-    const float bx = Pb.x, by = Pb.y, bz = Pb.z, bo = Pb.w;
-    const float cx = Pc.x, cy = Pc.y, cz = Pc.z, co = Pc.w;
-    const float bcx = fmaf(by, cz, -bz * cy), bcy = fmaf(bz, cx, -bx * cz), bcz = fmaf(bx, cy, -by * cx);
-    const float cax = fmaf(cy, az, -cz * ay), cay = fmaf(cz, ax, -cx * az), caz = fmaf(cx, ay, -cy * ax);
-    const float abx = fmaf(ay, bz, -az * by), aby = fmaf(az, bx, -ax * bz), abz = fmaf(ax, by, -ay * bx);
-    const float det = fmaf(ax, bcx, fmaf(ay, bcy, az * bcz));
-    const float inv = __frcp_rn(det);
-    x = fmaf(ao, bcx, fmaf(bo, cax, co * abx)) * inv;
-    y = fmaf(ao, bcy, fmaf(bo, cay, co * aby)) * inv;
-    z = fmaf(ao, bcz, fmaf(bo, caz, co * abz)) * inv;
-    // |q_k| = sqrt(2 o_k)
-    const float la = S.pfn[a], lb = S.pfn[b], lc = S.pfn[c];
-    const float H = la * lb * lc * fabsf(inv);  // P / |det| through the reciprocal (the factor 3 covers its ulp)
-    const float vn = fabsf(x) + fabsf(y) + fabsf(z);
-    const float u = 5.9604645e-8f;
-    err = 3.0f * u * H * (5.5f * (la + lb + lc) + 13.0f * vn);
-    // The analysis assumes no FP32 underflow or overflow: the numerators grow
-    // like |q|^4 and the determinant like |q|^3, so planes much nearer than
-    // 2^-28 or farther than 2^28 (tiny or huge boxes) are solved exactly.
-    const float qlo = fminf(la, fminf(lb, lc)), qhi = fmaxf(la, fmaxf(lb, lc));
-    if (!(u * H < 1e-3f) || !(err < 1e30f) || !(qlo >= 3.7252903e-9f) || !(qhi <= 268435456.0f))
-        err = __int_as_float(0x7f800000);  // +inf
 }
 
 // The rare exact paths of the filtered clipper, kept out of line so that the
@@ -845,33 +748,16 @@ __device__ void flush_batch(ClipSmem<PREC, CAP> &S, int &ncand, CellState &C, in
     __syncwarp();
 }
 
-// The main instance (CAP::BIG false) clips binned entry w of every warp; a
-// cell that overflows one of its lists goes to the retry list instead of
-// failing.  The large instance (one warp per block) clips entry retry[r] of
-// block r and writes its faces to overflow row r.
+// One cell: binned entry w.  The main instance (CAP::BIG false) writes its
+// faces to the cell's row; a cell that overflows one of its lists goes to the
+// retry list instead of failing.  The large instance writes to overflow row `row`.
 template <int PREC, class CAP, int SORT>
-__global__ void __maxnreg__(MM_CLIP_MAXNREG)
-k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sortedf, const int *__restrict__ start,
-       int64_t n,
-       const BoxDev *__restrict__ boxes, const int *__restrict__ cbox, double *__restrict__ vol,
-       double *__restrict__ cen, Slots sl, DevStatus *st, int collect, int cand_cap)
+__device__ __forceinline__ void
+clip_cell(ClipSmem<PREC, CAP> &S, const int64_t w, const bool strict, const int row, const int lane,
+          const double4_32a *__restrict__ sorted, const float4 *__restrict__ sortedf, const int *__restrict__ start,
+          int64_t n, const BoxDev *__restrict__ boxes, const int *__restrict__ cbox, double *__restrict__ vol,
+          double *__restrict__ cen, const Slots &sl, DevStatus *st, int collect, int cand_cap)
 {
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int64_t w;
-    bool strict = false;
-    if constexpr (CAP::BIG) {
-        const int nr = *(volatile int *)&st->nretry;
-        if (blockIdx.x == 0 && threadIdx.x == 0 && nr > sl.orows) atomicOr(&st->flags, ST_ECAP_RETRY);
-        if ((int64_t)blockIdx.x >= (nr < sl.orows ? (int64_t)nr : sl.orows)) return;
-        const int e = sl.retry[blockIdx.x];
-        strict = e < 0;
-        w = strict ? ~e : e;
-    } else {
-        w = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid;
-        if (w >= n) return;
-    }
-    ClipSmem<PREC, CAP> &S = reinterpret_cast<ClipSmem<PREC, CAP> *>(dyn_smem)[wid];
     // A box's cells occupy the same range of indices in the input order and in
     // the binned order (the bins are laid out box by box), so the box of
     // binned entry w is cbox[w]: no need to wait for the generator's id.
@@ -1070,7 +956,8 @@ k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorted
     // triangle (x, y, z) maps to that triangle and z, so the next vertex
     // around a face is one lookup.  Keys are unique in a closed
     // triangulation; the load stays below 3/4 (else the walk scans instead).
-    // The first triangle of each face is the lowest index containing it.
+    // A face starts at the triangle of its edge to the lowest plane slot (an
+    // order of the triangles that no schedule can change).
     constexpr int ETAB = CAP::ETAB, PB = CAP::PB, TB = CAP::TB;
     const bool use_tab = !C.err && 3 * C.nt <= (3 * ETAB) / 4;
     unsigned *etab = S.u.f.etab;
@@ -1093,7 +980,7 @@ k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorted
                 if (atomicCAS(&etab[h], 0xffffffffu, ent) == 0xffffffffu) break;
                 h = (h + 1) & (ETAB - 1);
             }
-            atomicMin(&first[x], t);
+            atomicMin(&first[x], (int)(y << 8) | t);
         }
         __syncwarp();
     }
@@ -1104,7 +991,7 @@ k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorted
             if (use_tab) {
                 const int f0 = first[p];
                 if (f0 != 0x7fffffff) {
-                    t0 = f0;
+                    t0 = f0 & 255;
                     const unsigned v = S.tv[t0];
                     const unsigned a = v & 255u, b = (v >> 8) & 255u, c = (v >> 16) & 255u;
                     y = a == (unsigned)p ? c : (b == (unsigned)p ? a : b);
@@ -1114,27 +1001,12 @@ k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorted
             }
             S.u.f.a[p] = 0.0;
             if (t0 < 0) continue;  // plane no longer bounds the cell
-            // Fan about the polygon's first vertex v0 with offsets d = v - v0
-            // formed once per vertex.  The offsets lie in the plane x.q = o,
-            // so d_a x d_b is parallel to q and q . (d_a x d_b) equals
-            // (|q|^2 / q_k) times the 2-D cross product of the two coordinates
-            // other than k, the axis where |q| is largest.  Edge (a, b) spans
-            // the triangle (v0, a, b) with 2-D weight w; with W = sum w:
-            // area = |W| |q| / (2 |q_k|), pyramid volume A |q| / 6 =
-            // |W| |q|^2 / (12 |q_k|), centroid offset = sum w (d_a + d_b) / (3 W)
-            // in the two kept coordinates, and in the k-th from the plane
-            // equation q . offset = 0.  Offsets from v0 keep the rounding
-            // relative to the face's own size.
             const double qx = S.px[p], qy = S.py[p], qz = S.pz[p];
-            const long long aqx = abs_bits(qx), aqy = abs_bits(qy), aqz = abs_bits(qz);
-            const int k = (aqx >= aqy && aqx >= aqz) ? 0 : (aqy >= aqz ? 1 : 2);
+            const int k = fan_axis(qx, qy, qz);
             const double *T1 = k == 0 ? S.ty : S.tx;  // kept coordinates (u, v)
             const double *T2 = k == 2 ? S.ty : S.tz;
-            const double qk = k == 0 ? qx : (k == 1 ? qy : qz);
-            const double q1 = k == 0 ? qy : qx, q2 = k == 2 ? qy : qz;
             const double u0 = T1[t0], v0 = T2[t0];
-            double au = 0.0, av = 0.0;  // offset of the current vertex
-            double W = 0.0, su = 0.0, sv = 0.0;
+            FaceFan F;
             int cnt = 0;
             bool ok = false;
             for (int guard = 0; guard < CAP::TM; ++guard) {
@@ -1160,38 +1032,20 @@ k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorted
                 if (tn < 0) break;
                 ++cnt;
                 if (tn == t0) { ok = true; break; }
-                const double bu = T1[tn] - u0, bv = T2[tn] - v0;
-                const double w = au * bv - av * bu;
-                W += w;
-                su += w * (au + bu);
-                sv += w * (av + bv);
-                au = bu; av = bv;
+                F.edge(T1[tn] - u0, T2[tn] - v0);
                 y = z;
             }
             fan += cnt;
             if (!ok) { C.err |= ST_EDEGEN_CUT; continue; }
-            const double aw = fabs(W);
-            const double qn2 = 2.0 * S.po[p];  // |q|^2
-            // 1 / q_k and 1 / (3 W) from one reciprocal of 3 W q_k; a face
-            // of zero fan weight (area 0) takes 0 for both
-            const double w3 = 3.0 * W;
-            const bool nz = abs_bits(W) != 0;
-            const double r = nz ? 1.0 / (w3 * qk) : 0.0;
-            const double iq = w3 * r, iqk = fabs(iq);
-            const double area = 0.5 * aw * (qn2 * rsqrt(qn2)) * iqk;
-            const double i3w = qk * r;
-            const double du = su * i3w, dv = sv * i3w;
-            const double dk = -(q1 * du + q2 * dv) * iq;
-            const double fx = S.tx[t0] + (k == 0 ? dk : du);
-            const double fy = S.ty[t0] + (k == 1 ? dk : (k == 0 ? du : dv));
-            const double fz = S.tz[t0] + (k == 2 ? dk : dv);
+            double area, fx, fy, fz, vp;
+            face_of_fan(F, k, qx, qy, qz, S.po[p], S.tx[t0], S.ty[t0], S.tz[t0], area, fx, fy, fz, vp);
             S.u.f.a[p] = area;
             S.u.f.x[p] = fx; S.u.f.y[p] = fy; S.u.f.z[p] = fz;
-            const double vp = aw * qn2 * iqk * (1.0 / 12.0);
             vl += vp;
-            vcx += 0.75 * vp * fx;
-            vcy += 0.75 * vp * fy;
-            vcz += 0.75 * vp * fz;
+            const double vw = 0.75 * vp;
+            vcx = __fma_rn(vw, fx, vcx);
+            vcy = __fma_rn(vw, fy, vcy);
+            vcz = __fma_rn(vw, fz, vcz);
         }
         C.err = __reduce_or_sync(FULL, (unsigned)C.err);
     }
@@ -1208,7 +1062,7 @@ k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorted
         unsigned char *const rsh = CAP::BIG ? sl.osh : sl.sh;
         double *const rarea = CAP::BIG ? sl.oarea : sl.area;
         double *const rfc = CAP::BIG ? sl.ofc : sl.fc;
-        const int64_t sbase = CAP::BIG ? (int64_t)blockIdx.x * CAP::MF : (int64_t)self * CAP::MF;
+        const int64_t sbase = CAP::BIG ? (int64_t)row * CAP::MF : (int64_t)self * CAP::MF;
         const int64_t ns = CAP::BIG ? sl.orows * (int64_t)CAP::MF : n * (int64_t)CAP::MF;
         for (int p0 = 0; p0 < C.np; p0 += 32) {
             const int p = p0 + lane;
@@ -1243,8 +1097,8 @@ k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorted
             }
         }
         if constexpr (CAP::BIG) {
-            sl.ocnt[blockIdx.x] = nface;
-            sl.cnt[self] = C.err ? 0 : -(int)blockIdx.x - 1;
+            sl.ocnt[row] = nface;
+            sl.cnt[self] = C.err ? 0 : -row - 1;
         } else {
             sl.cnt[self] = nface;
         }
@@ -1268,10 +1122,42 @@ k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorted
     }
 }
 
+// The main instance clips one binned entry per warp, or, with a list, its
+// *list_n entries, warps taking them in turn.  The large instance (one warp per
+// block) clips entry retry[r] of block r and writes its faces to overflow row r.
+template <int PREC, class CAP, int SORT>
+__global__ void __maxnreg__(MM_CLIP_MAXNREG)
+k_clip(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sortedf, const int *__restrict__ start,
+       int64_t n,
+       const BoxDev *__restrict__ boxes, const int *__restrict__ cbox, double *__restrict__ vol,
+       double *__restrict__ cen, Slots sl, DevStatus *st, int collect, int cand_cap, const int *__restrict__ list,
+       const int *__restrict__ list_n)
+{
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    ClipSmem<PREC, CAP> &S = reinterpret_cast<ClipSmem<PREC, CAP> *>(dyn_smem)[wid];
+    if constexpr (CAP::BIG) {
+        const int nr = *(volatile int *)&st->nretry;
+        if (blockIdx.x == 0 && threadIdx.x == 0 && nr > sl.orows) atomicOr(&st->flags, ST_ECAP_RETRY);
+        if ((int64_t)blockIdx.x >= (nr < sl.orows ? (int64_t)nr : sl.orows)) return;
+        const int e = sl.retry[blockIdx.x];
+        clip_cell<PREC, CAP, SORT>(S, e < 0 ? ~e : e, e < 0, (int)blockIdx.x, lane, sorted, sortedf, start, n, boxes,
+                                   cbox, vol, cen, sl, st, collect, cand_cap);
+    } else {
+        const int64_t count = list ? (int64_t)*list_n : n, step = (int64_t)gridDim.x * (blockDim.x >> 5);
+        for (int64_t e = (int64_t)blockIdx.x * (blockDim.x >> 5) + wid; e < count; e += step) {
+            clip_cell<PREC, CAP, SORT>(S, list ? (int64_t)list[e] : e, false, 0, lane, sorted, sortedf, start, n, boxes,
+                                       cbox, vol, cen, sl, st, collect, cand_cap);
+            __syncwarp();
+        }
+    }
+}
+
 template <int PREC, class CAP, int SORT>
 static void launch_clip_t(const double4_32a *sorted, const float4 *sortedf, const int *start, int64_t n,
                           const BoxDev *boxes, const int *cbox, double *vol, double *cen, Slots sl, DevStatus *st,
-                          int collect, int warps, int cand_cap, int64_t blocks, cudaStream_t s)
+                          int collect, int warps, int cand_cap, int64_t blocks, const int *list,
+                          const int *list_n, cudaStream_t s)
 {
     static bool configured = false;  // the attribute is per function and process-wide
     if (!configured) {
@@ -1281,24 +1167,26 @@ static void launch_clip_t(const double4_32a *sorted, const float4 *sortedf, cons
     }
     const size_t smem = sizeof(ClipSmem<PREC, CAP>) * warps;
     k_clip<PREC, CAP, SORT><<<(unsigned)blocks, 32 * warps, smem, s>>>(sorted, sortedf, start, n, boxes, cbox, vol, cen,
-                                                                 sl, st, collect, cand_cap);
+                                                                 sl, st, collect, cand_cap, list, list_n);
 }
 
 void launch_clip(const double4_32a *sorted, const float4 *sortedf, const int *start, int64_t n, const BoxDev *boxes,
                  const int *cbox,
                  int precision, int collect, int warps, int cand_cap, int sort, double *vol, double *cen,
-                 Slots sl, DevStatus *st, cudaStream_t s)
+                 Slots sl, DevStatus *st, const int *list, const int *list_n, cudaStream_t s)
 {
     warps = warps < 1 ? 1 : (warps > CLIP_MAX_WARPS ? CLIP_MAX_WARPS : warps);
     cand_cap = cand_cap < 32 ? 32 : (cand_cap > CBATCH ? CBATCH : cand_cap);
-    const int64_t nb = (n + warps - 1) / warps;
+    // a list holds few cells: enough blocks to spread a few thousand over the chip
+    int64_t nb = (n + warps - 1) / warps;
+    if (list && nb > 1216) nb = 1216;
     // the sort variant only changes speed, so the direct FP64 clipper keeps one
     if (precision == 0)
-        launch_clip_t<0, CapMain, 0>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, warps, cand_cap, nb, s);
+        launch_clip_t<0, CapMain, 0>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, warps, cand_cap, nb, list, list_n, s);
     else if (sort == 1)
-        launch_clip_t<1, CapMain, 1>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, warps, cand_cap, nb, s);
+        launch_clip_t<1, CapMain, 1>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, warps, cand_cap, nb, list, list_n, s);
     else
-        launch_clip_t<1, CapMain, 0>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, warps, cand_cap, nb, s);
+        launch_clip_t<1, CapMain, 0>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, warps, cand_cap, nb, list, list_n, s);
 }
 
 void launch_clip_big(const double4_32a *sorted, const float4 *sortedf, const int *start, int64_t n,
@@ -1308,9 +1196,9 @@ void launch_clip_big(const double4_32a *sorted, const float4 *sortedf, const int
     if (sl.orows < 1) return;
     cand_cap = cand_cap < 32 ? 32 : (cand_cap > CBATCH ? CBATCH : cand_cap);
     if (precision == 0)
-        launch_clip_t<0, CapBig, 0>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, 1, cand_cap, sl.orows, s);
+        launch_clip_t<0, CapBig, 0>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, 1, cand_cap, sl.orows, nullptr, nullptr, s);
     else
-        launch_clip_t<1, CapBig, 0>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, 1, cand_cap, sl.orows, s);
+        launch_clip_t<1, CapBig, 0>(sorted, sortedf, start, n, boxes, cbox, vol, cen, sl, st, collect, 1, cand_cap, sl.orows, nullptr, nullptr, s);
 }
 
 }  // namespace mm

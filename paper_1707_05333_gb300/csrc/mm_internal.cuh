@@ -25,6 +25,12 @@ constexpr int MAXF = 48;    // faces written per cell
 constexpr int MAXRING = 48; // search rings before giving up
 constexpr int PMAX_BIG = 128, TMAX_BIG = 256, NSTAGE_BIG = 64, MAXF_BIG = 128, MAXRING_BIG = 128;
 constexpr int CLIP_MAX_WARPS = 8;  // warps (cells) per block of the clipper, tunable at run time
+// Cells from which the grouped clipper (mm_cells.cu) runs.  Below, the chip is
+// not full and a warp per cell finishes sooner.  Tessellation, warp per cell
+// against grouped: 1000 random generators 0.29 / 0.40 ms, 4100 0.43 / 0.60,
+// 8000 0.65 / 0.65, 16000 0.99 / 0.87, 200003 9.5 / 5.4; jittered lattices 20^3
+// 0.38 / 0.28, 64^3 6.4 / 3.6.
+constexpr int64_t CELLS_MIN = 8000;
 // Overflow rows reserved when the count of retried cells is not known in
 // advance (graph mode); mm_tessellate sizes them to the count it reads.
 constexpr int RETRY_ROWS_FIXED = 256;
@@ -60,6 +66,7 @@ struct DevStatus {
     unsigned long long fan64;    // FP64 fan terms of the face geometry
     unsigned long long tested;   // candidates tested against the cell
     int nretry;                  // cells sent to the large clipper
+    int nlist;                   // cells the grouped clipper leaves to the warp-per-cell one
 };
 
 // One periodic box of a batch.
@@ -110,14 +117,19 @@ void launch_scan(const int *in, int *out, int64_t n, int *tmp, cudaStream_t s);
 
 // vol receives each cell's volume and cen its first moment about the
 // generator ([3][n]); launch_face_write turns the moment into the centroid.
-// The main clipper (every cell, fixed capacities; a cell over a capacity is
-// appended to sl.retry) and the large clipper (the cells of sl.retry, their
+// The main clipper (every cell, or the cells of a list; a cell over one of its
+// fixed capacities is appended to sl.retry) and the large clipper (the cells of sl.retry, their
 // faces to the overflow rows; a launch of sl.orows warps handles the first
 // min(nretry, orows) of them and flags the rest).
 void launch_clip(const double4_32a *sorted, const float4 *sortedf, const int *start, int64_t n, const BoxDev *boxes,
                  const int *cbox,
                  int precision, int collect, int warps, int cand_cap, int sort, double *vol, double *cen,
-                 Slots sl, DevStatus *st, cudaStream_t s);
+                 Slots sl, DevStatus *st, const int *list, const int *list_n, cudaStream_t s);
+// The grouped clipper (mm_cells.cu): every cell; those it leaves are appended
+// to list (room for n) and counted in *list_n.
+void launch_cells(const double4_32a *sorted, const float4 *sortedf, const int *start, int64_t n, const BoxDev *boxes,
+                  const int *cbox, int cand_cap, double *vol, double *cen, Slots sl, int *list, int *list_n,
+                  cudaStream_t s);
 void launch_clip_big(const double4_32a *sorted, const float4 *sortedf, const int *start, int64_t n,
                      const BoxDev *boxes, const int *cbox, int precision, int collect, int cand_cap, double *vol,
                      double *cen, Slots sl, DevStatus *st, cudaStream_t s);
