@@ -491,7 +491,7 @@ static mm_status tess_enqueue(mm_ctx *c, const double *pos, bool fixed)
         list = P<int>(c->emit_cnt);
         launch_cells(P<double4_32a>(c->sorted), P<float4>(c->sortedf), P<int>(c->bin_start), n, boxes, cbox,
                      c->cfg.cand_cap, P<double>(c->vol), P<double>(c->cen), sl, list, &c->st->nlist, s);
-        c->launches += 2;
+        c->launches += 1;
     }
     launch_clip(P<double4_32a>(c->sorted), P<float4>(c->sortedf), P<int>(c->bin_start), n, boxes, cbox, prec,
                 c->cfg.collect_stats,

@@ -1,25 +1,27 @@
-// mm_cells.cu -- the filtered clipper for ordinary cells, in two kernels.
+// mm_cells.cu -- the filtered clipper for ordinary cells.
 //
 // The same cell construction as k_clip (mm_clip.cu), with the same decisions,
 // the same plane order and the same FP64 geometry bit for bit, laid out for
-// the usual cell of 10-30 faces.  k_cells clips with G lanes a cell: 32/G
+// the usual cell of 10-30 faces.  Cells are clipped with G lanes each: 32/G
 // cells share a warp, so the control, ballots and topology updates of one
 // instruction stream serve 32/G cells, and a cut's handful of removed and new
-// vertices fill the G lanes instead of a fraction of 32.  It leaves each cell
-// as plane references and triangles; k_cell_geom forms the FP64 geometry with
-// full warps.
+// vertices fill the G lanes instead of a fraction of 32.  Then the warp forms
+// the FP64 geometry of its cells together, with full lanes (warp_geometry).
 //
-// What bounds them and what they measured (GB300, jittered 64^3 lattice and
+// What bounds it and what it measured (GB300, jittered 64^3 lattice and
 // 200003 random generators, ncu durations; k_clip took 5.89 and 8.89 ms):
-//  * k_cells 1.70 and 3.58 ms: issue slots and dependent latencies (2.1
-//    instructions a cycle, 4320 a cell against k_clip's 14200; 15 warps an SM,
-//    limited by 3.4 KB of shared memory a cell and 128 registers).  Loops are
-//    kept rolled: unrolled, the body outgrew the instruction cache and half of
-//    the cycles went to fetching it (5.3 and 13.0 ms).
-//  * k_cell_geom 1.45 and 1.10 ms: the FP64 pipe (84 % busy, 91 FP64
-//    instructions a cell against 236 inside k_clip, whose lanes were a third full).
+// 2.77 and 4.28 ms, of dependent latencies with 15 warps an SM (3.4 KB of
+// shared memory a cell, 128 registers): 1.6 instructions a cycle, 5340 a cell
+// against k_clip's 14200, and the FP64 pipe 51 % busy with 106 instructions a
+// cell against 236.
+//  * Loops are kept rolled: unrolled, the body outgrew the instruction cache
+//    and half of the cycles went to fetching it (5.3 and 13.0 ms).
 //  * Screening candidates a lane each after the first 16 instead of trying all
-//    one by one: random generators 4.33 -> 3.58 ms.
+//    one by one: random generators 4.33 -> 3.58 ms (clipping alone).
+//  * The geometry as a kernel of its own (1.45 and 1.10 ms, FP64 pipe 84 %
+//    busy, after 1.70 and 3.58 ms of clipping) left the FP64 pipe idle in one
+//    kernel and the issue slots in the other: 3.15 and 4.68 ms in all, here
+//    2.88 and 4.33 before the shorter FP64 sequences (mm_fp64.cuh, solve64).
 //
 // A cell that outgrows these lists (more than 32 live planes, 48 vertices, 32
 // new vertices in a cut, CELL_RINGS search rings), holds a coincident
@@ -41,12 +43,6 @@ constexpr int LANES = 8;   // lanes a cell (16 lanes: jittered 64^3 2.35 ms for 
 constexpr unsigned BOX_PLANE = 31u << 27;  // plane reference of box face k: BOX_PLANE | k
 constexpr unsigned IDX_MASK = 0x7ffffffu;  // sorted index of a plane reference (MM_MAX_CELLS < 2^27)
 static_assert(MM_MAX_CELLS < (1LL << 27), "a plane reference holds the index in 27 bits");
-
-// What k_cells leaves for k_cell_geom, in the cell's row of the area slots:
-// word 0: planes | vertices << 8 (0: the cell went to the list), then the CPM
-// plane references, then the vertices' triangles, two to a word.
-constexpr int REC_TRI = 1 + CPM;
-static_assert((REC_TRI + CTM / 2) * 4 <= MAXF * 8, "the record fits the row");
 
 struct __align__(16) CellSmem {
     float4 tf[CTM];       // vertex; .w = error bound (upper 16 bits, rounded up) | a | b << 5 | c << 10
@@ -302,11 +298,287 @@ __device__ __forceinline__ bool sort_batch(CellSmem &S, int m, unsigned base, in
     return tie;
 }
 
+// ---------------------------------------------------------------------------
+// Geometry of a warp's cells once they are clipped.  Their planes, vertices
+// and faces are spread over the 32 lanes as flat lists, because an FP64
+// instruction occupies the pipe for the same 16 cycles whatever the number of
+// active lanes: the FP64 work per cell is that of full warps.  Faces are taken
+// in the order of their number of vertices, so that the lanes of a warp walk
+// polygons of like length.
+// ---------------------------------------------------------------------------
+constexpr int GC = 32 / LANES;   // cells of a warp
+constexpr int GV = 176;          // vertices of one pass (4 cells of 27; a fuller warp takes two passes)
+constexpr int GP = 96;           // planes of one pass (4 cells of 16)
+constexpr int TEAM = LANES;      // lanes of one cell
+static_assert(GV >= CTM && GP >= CPM, "any one cell fits a pass");
+
+struct __align__(16) GeomSmem {
+    double vx[GV], vy[GV], vz[GV];
+    double px[GP], py[GP], pz[GP], po[GP];  // planes, then face area and centroid
+    double vp[GP];                          // pyramid volumes
+    double off[GC][9];
+    unsigned ref[GC][CPM];
+    unsigned live[GC];                      // slots with a face
+    int vbase[GC], pbase[GC];               // first vertex and plane of a cell in the lists
+    int hist[16];
+    unsigned short tri[GC][CTM];
+    unsigned short item[GP], order[GP];     // cell << 5 | slot of a plane; planes by number of vertices
+    unsigned short vitem[GV];               // cell << 6 | vertex
+    unsigned char nxt[GP][CPM];             // vertex of the cell holding the directed edge plane -> slot
+    unsigned char deg[GP];
+    unsigned char bad[GC];
+};
+static_assert(sizeof(GeomSmem) <= GC * sizeof(CellSmem), "it takes the place of the clipped cells");
+
+__device__ __forceinline__ int plane_of(const GeomSmem &S, int c, unsigned slot)
+{
+    return S.pbase[c] + __popc(S.live[c] & ((1u << slot) - 1u));
+}
+
+// S holds the cells' references, triangles, offsets and live slots; w0 is the
+// warp's first cell, nt this lane's cell's vertices (0: none to form).
+__device__ __forceinline__ void
+warp_geometry(GeomSmem &S, int lane, int64_t w0, int w, int nt, const BoxDev *gp, int self,
+              const double4_32a *__restrict__ sorted, int64_t n, const BoxDev *__restrict__ boxes,
+              const int *__restrict__ cbox, double *__restrict__ vol, double *__restrict__ cen, const Slots &sl,
+              int *__restrict__ list, int *__restrict__ list_n)
+{
+    const int tc = lane / TEAM, tl = lane % TEAM;
+    const int64_t sbase = (int64_t)self * MAXF, ns = n * (int64_t)MAXF;
+    bool todo = nt > 0;
+    while (__any_sync(FULL, todo)) {
+        // ---- the cells of this pass: as many, in order, as the lists hold
+        const int nl = __popc(S.live[tc]);
+        int vb = todo && tl == 0 ? nt : 0, pb = todo && tl == 0 ? nl : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(FULL, vb, o), p = __shfl_up_sync(FULL, pb, o);
+            if (lane >= o) { vb += v; pb += p; }
+        }
+        const bool mine = todo && vb <= GV && pb <= GP;  // prefix sums: true for a first run of the cells left
+        const int nv = __reduce_max_sync(FULL, mine ? vb : 0), npl = __reduce_max_sync(FULL, mine ? pb : 0);
+        vb -= nt;
+        pb -= nl;
+        if (mine && tl == 0) { S.vbase[tc] = vb; S.pbase[tc] = pb; }
+        if (mine) {
+            const unsigned lv = S.live[tc];
+#pragma unroll 1
+            for (unsigned r = lv; r; r &= r - 1u) {
+                const int p = __ffs((int)r) - 1, k = pb + __popc(lv & ((1u << p) - 1u));
+                if ((k & (TEAM - 1)) == tl) S.item[k] = (unsigned short)(tc << 5 | p);
+            }
+#pragma unroll 2
+            for (int t = tl; t < nt; t += TEAM) S.vitem[vb + t] = (unsigned short)(tc << 6 | t);
+        }
+        if (lane < 16) S.hist[lane] = 0;
+        {
+            uint4 *const z = reinterpret_cast<uint4 *>(&S.nxt[0][0]);
+#pragma unroll 2
+            for (int i = lane; i < npl * CPM / 16; i += 32) z[i] = make_uint4(FULL, FULL, FULL, FULL);
+        }
+        __syncwarp();
+        // ---- planes and edges
+#pragma unroll 1
+        for (int k = lane; k < npl; k += 32) {
+            const int it = S.item[k], c = it >> 5;
+            double x, y, z, o;
+            plane64(S.off[c], S.ref[c][it & 31], sorted, boxes + cbox[w0 + c], x, y, z, o);
+            S.px[k] = x; S.py[k] = y; S.pz[k] = z; S.po[k] = o;
+            S.vp[k] = 0.0;
+        }
+#pragma unroll 1
+        for (int k = lane; k < nv; k += 32) {
+            const int it = S.vitem[k], c = it >> 6, t = it & 63;
+            const unsigned v = S.tri[c][t], x = v & 31u, y = (v >> 5) & 31u, z = v >> 10;
+            S.nxt[plane_of(S, c, x)][y] = (unsigned char)t;
+            S.nxt[plane_of(S, c, y)][z] = (unsigned char)t;
+            S.nxt[plane_of(S, c, z)][x] = (unsigned char)t;
+        }
+        __syncwarp();
+        // ---- vertices; an edge two triangles claim is not a closed cell
+#pragma unroll 1
+        for (int k = lane; k < nv; k += 32) {
+            const int it = S.vitem[k], c = it >> 6, t = it & 63;
+            const unsigned v = S.tri[c][t], x = v & 31u, y = (v >> 5) & 31u, z = v >> 10;
+            const int a = plane_of(S, c, x), b = plane_of(S, c, y), d = plane_of(S, c, z);
+            if (S.nxt[a][y] != t || S.nxt[b][z] != t || S.nxt[d][x] != t) S.bad[c] = 1;
+            vertex64(S, a, b, d, S.vx[k], S.vy[k], S.vz[k]);
+        }
+        // ---- faces by number of vertices: the bytes of the edge row in use
+#pragma unroll 1
+        for (int k = lane; k < npl; k += 32) {
+            const uint4 *const r = reinterpret_cast<const uint4 *>(S.nxt[k]);
+            const uint4 a = r[0], b = r[1];
+            const unsigned u = ~a.x & 0x80808080u, v = ~a.y & 0x80808080u, x = ~a.z & 0x80808080u, y = ~a.w & 0x80808080u;
+            const unsigned u2 = ~b.x & 0x80808080u, v2 = ~b.y & 0x80808080u, x2 = ~b.z & 0x80808080u, y2 = ~b.w & 0x80808080u;
+            const int d = min(__popc(u | v >> 1 | x >> 2 | y >> 3 | u2 >> 4 | v2 >> 5 | x2 >> 6 | y2 >> 7), 15);
+            S.deg[k] = (unsigned char)d;
+            atomicAdd(&S.hist[d], 1);
+        }
+        __syncwarp();
+        {
+            const int h = lane < 16 ? S.hist[15 - lane] : 0;  // most vertices first
+            int p = h;
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) {
+                const int q = __shfl_up_sync(FULL, p, o);
+                if (lane >= o) p += q;
+            }
+            if (lane < 16) S.hist[15 - lane] = p - h;
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int k = lane; k < npl; k += 32) S.order[atomicAdd(&S.hist[S.deg[k]], 1)] = (unsigned short)k;
+        __syncwarp();
+#pragma unroll 1
+        for (int j = lane; j < npl; j += 32) {
+            const int k = S.order[j], it = S.item[k], c = it >> 5;
+            const unsigned p = it & 31;
+            const int vbc = S.vbase[c];
+            // the walk starts at the vertex holding the edge to the lowest slot
+            unsigned y = 0;
+            int t0 = 255;
+            {
+                const uint4 *const r = reinterpret_cast<const uint4 *>(S.nxt[k]);
+                const uint4 a = r[0], b = r[1];
+                const unsigned wv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int q = 7; q >= 0; --q) {
+                    const unsigned u = ~wv[q] & 0x80808080u;
+                    if (u) {
+                        const int s = __ffs((int)u) >> 3;  // byte 0..3 (its bit 7 is set)
+                        y = (unsigned)(4 * q + s - 1);
+                        t0 = (int)((wv[q] >> (8 * (s - 1))) & 255u);
+                    }
+                }
+            }
+            const double qx = S.px[k], qy = S.py[k], qz = S.pz[k];
+            const int ka = fan_axis(qx, qy, qz);
+            const double *T1 = (ka == 0 ? S.vy : S.vx) + vbc, *T2 = (ka == 2 ? S.vy : S.vz) + vbc;
+            const double u0 = T1[t0], v0 = T2[t0];
+            FaceFan F;
+            bool ok = false, any = false;
+#pragma unroll 1
+            for (int guard = 0; guard < CTM; ++guard) {
+                const unsigned vt = S.tri[c][guard == 0 ? t0 : (int)S.nxt[k][y]];
+                y = (vt & 31u) ^ ((vt >> 5) & 31u) ^ (vt >> 10) ^ p ^ y;
+                const int tn = S.nxt[k][y];
+                if (tn == 255) break;
+                if (tn == t0) { ok = true; break; }
+                const double bu = T1[tn] - u0, bv = T2[tn] - v0;
+                if (any) F.edge(bu, bv);
+                else F.begin(bu, bv);
+                any = true;
+            }
+            if (!ok) S.bad[c] = 1;
+            double area, fx, fy, fz, vp;
+            face_of_fan(F, ka, qx, qy, qz, S.po[k], S.vx[vbc + t0], S.vy[vbc + t0], S.vz[vbc + t0], area, fx, fy, fz, vp);
+            S.px[k] = area; S.py[k] = fx; S.pz[k] = fy; S.po[k] = fz;
+            S.vp[k] = vp;
+        }
+        __syncwarp();
+        // ---- slots, cell by cell in order of the planes
+        const double amin = gp->amin;
+        int nface = 0;
+        {
+            const int nout = mine && !S.bad[tc] ? nl : 0, maxout = __reduce_max_sync(FULL, nout);
+#pragma unroll 1
+            for (int i = tl; i - tl < maxout; i += TEAM) {
+                const int k = pb + i;
+                double area = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
+                if (i < nout) {
+                    // the first moment takes the centroid's place
+                    const double vw = __dmul_rn(0.75, S.vp[k]);
+                    area = S.px[k]; fx = S.py[k]; fy = S.pz[k]; fz = S.po[k];
+                    S.py[k] = __dmul_rn(vw, fx);
+                    S.pz[k] = __dmul_rn(vw, fy);
+                    S.po[k] = __dmul_rn(vw, fz);
+                }
+                const bool keep = i < nout && abs_bits(area) > abs_bits(amin);
+                const unsigned km = (__ballot_sync(FULL, keep) >> (tc * TEAM)) & ((1u << TEAM) - 1u);
+                if (keep) {
+                    const int64_t s = sbase + nface + __popc(km & ((1u << tl) - 1u));
+                    const unsigned ref = S.ref[tc][S.item[k] & 31], code = ref >> 27;
+                    int nb = self, sh;
+                    if (code == 31u) {
+                        const int kf = (int)(ref & 7u), d = kf >> 1, e = d == 0 ? 1 : (d == 1 ? 3 : 9);
+                        sh = 13 + ((kf & 1) ? -e : e);
+                    } else {
+                        nb = (int)__double_as_longlong(sorted[ref & IDX_MASK].w);
+                        sh = (int)code;
+                    }
+                    sl.nb[s] = nb;
+                    sl.sh[s] = (unsigned char)sh;
+                    sl.area[s] = area;
+                    sl.fc[s] = fx;
+                    sl.fc[ns + s] = fy;
+                    sl.fc[2 * ns + s] = fz;
+                }
+                nface += __popc(km);
+            }
+        }
+        __syncwarp();
+        // ---- volume and first moment: k_clip's tree over the 32 slots (p and
+        // p + 16, then p + 8, p + 4, p + 2, p + 1; a slot without a face adds 0)
+        double a0, a1, a2, a3;
+        {
+            const unsigned lv = S.live[tc];
+            double b[2][4];
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                double s[2][4];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int p = tl + 8 * g + 16 * e;
+                    const bool has = mine && ((lv >> p) & 1u);
+                    const int k = has ? pb + __popc(lv & ((1u << p) - 1u)) : 0;
+                    s[e][0] = has ? S.vp[k] : 0.0;
+                    s[e][1] = has ? S.py[k] : 0.0;
+                    s[e][2] = has ? S.pz[k] : 0.0;
+                    s[e][3] = has ? S.po[k] : 0.0;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) b[g][q] = __dadd_rn(s[0][q], s[1][q]);
+            }
+            a0 = __dadd_rn(b[0][0], b[1][0]);
+            a1 = __dadd_rn(b[0][1], b[1][1]);
+            a2 = __dadd_rn(b[0][2], b[1][2]);
+            a3 = __dadd_rn(b[0][3], b[1][3]);
+        }
+        // each exchange halves the sums a lane keeps: lanes 0-1 of the eight end
+        // with the volume, 2-3, 4-5 and 6-7 with the moment's components
+        static_assert(TEAM == 8, "three exchanges");
+        {
+            const bool h4 = (tl & 4) != 0, h2 = (tl & 2) != 0;
+            double k0 = h4 ? a2 : a0, k1 = h4 ? a3 : a1;
+            const double s0 = h4 ? a0 : a2, s1 = h4 ? a1 : a3;
+            k0 += __shfl_xor_sync(FULL, s0, 4);
+            k1 += __shfl_xor_sync(FULL, s1, 4);
+            double q = h2 ? k1 : k0;
+            q += __shfl_xor_sync(FULL, h2 ? k0 : k1, 2);
+            q += __shfl_xor_sync(FULL, q, 1);
+            a0 = q;
+        }
+        if (mine && (tl & 1) == 0) {
+            if (S.bad[tc]) {
+                if (tl == 0) list[atomicAdd(list_n, 1)] = w;
+            } else if (tl == 0) {
+                sl.cnt[self] = nface;
+                vol[self] = a0;
+            } else {
+                cen[(tl / 2 - 1) * n + self] = a0;
+            }
+        }
+        todo = todo && !mine;
+        __syncwarp();
+    }
+}
+
 template <int G>
 __global__ void __launch_bounds__(64, 8)
 k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sortedf, const int *__restrict__ start,
-        int64_t n, const BoxDev *__restrict__ boxes, const int *__restrict__ cbox, Slots sl, int cand_cap,
-        int *__restrict__ list, int *__restrict__ list_n)
+        int64_t n, const BoxDev *__restrict__ boxes, const int *__restrict__ cbox, double *__restrict__ vol,
+        double *__restrict__ cen, Slots sl, int cand_cap, int *__restrict__ list, int *__restrict__ list_n)
 {
     constexpr int CPW = 32 / G;
     constexpr unsigned GM = (1u << G) - 1u;
@@ -729,322 +1001,43 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
         __syncwarp();
     }
 
-    // ---- the record
-    if (wi < n) {
-        const int self = (int)__double_as_longlong(sorted[w].w);
-        unsigned *const row = reinterpret_cast<unsigned *>(sl.area + (int64_t)self * MAXF);
-        if (gl == 0) {
-            row[0] = bad ? 0u : (unsigned)np | ((unsigned)nt << 8);
-            if (bad) list[atomicAdd(list_n, 1)] = w;
-        }
-        if (!bad) {
-#pragma unroll 1
-            for (int p = gl; p < np; p += G) row[1 + p] = S.pid[p];
-#pragma unroll 1
-            for (int t = 2 * gl; t < nt; t += 2 * G)
-                row[REC_TRI + (t >> 1)] = tri_of(S.tf[t].w) | (t + 1 < nt ? tri_of(S.tf[t + 1].w) << 16 : 0u);
-        }
+    // ---- the cells' topology, in the same memory, and their geometry
+    const int self = (int)__double_as_longlong(sorted[w].w);
+    if (wi >= n) nt = 0;
+    if (bad && nt > 0) {
+        if (gl == 0) list[atomicAdd(list_n, 1)] = w;
+        nt = 0;
     }
-}
-
-// ---------------------------------------------------------------------------
-// Geometry of the cells k_cells clipped.  A warp takes GC cells and spreads
-// their planes, vertices and faces over its lanes as flat lists, because an
-// FP64 instruction occupies the pipe for the same 16 cycles whatever the
-// number of active lanes: the FP64 work per cell is that of full warps.  Faces
-// are taken in the order of their number of vertices, so that the lanes of a
-// warp walk polygons of like length.
-// ---------------------------------------------------------------------------
-constexpr int GC = 8;            // cells of a warp
-constexpr int GV = 304;          // vertices of one pass (8 cells of 27; a fuller warp takes two passes)
-constexpr int GP = 176;          // planes of one pass
-constexpr int TEAM = 32 / GC;    // lanes that load one cell
-static_assert(GV >= CTM && GP >= CPM, "any one cell fits a pass");
-
-struct __align__(16) GeomSmem {
-    double vx[GV], vy[GV], vz[GV];
-    double px[GP], py[GP], pz[GP], po[GP];  // planes, then face area and centroid
-    double vp[GP];                          // pyramid volumes
-    double off[GC][9];
-    unsigned ref[GC][CPM];
-    unsigned live[GC];                      // slots with a face
-    int vbase[GC], pbase[GC];               // first vertex and plane of a cell in the lists
-    int hist[16];
-    unsigned short tri[GC][CTM];
-    unsigned short item[GP], order[GP];     // cell << 5 | slot of a plane; planes by number of vertices
-    unsigned short vitem[GV];               // cell << 6 | vertex
-    unsigned char nxt[GP][CPM];             // vertex of the cell holding the directed edge plane -> slot
-    unsigned char deg[GP];
-    unsigned char bad[GC];
-};
-
-__device__ __forceinline__ int plane_of(const GeomSmem &S, int c, unsigned slot)
-{
-    return S.pbase[c] + __popc(S.live[c] & ((1u << slot) - 1u));
-}
-
-__global__ void __launch_bounds__(32)
-k_cell_geom(const double4_32a *__restrict__ sorted, int64_t n, const BoxDev *__restrict__ boxes,
-            const int *__restrict__ cbox, double *__restrict__ vol, double *__restrict__ cen, Slots sl,
-            int *__restrict__ list, int *__restrict__ list_n)
-{
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
-    GeomSmem &S = *reinterpret_cast<GeomSmem *>(dyn_smem);
-    const int lane = threadIdx.x, tc = lane / TEAM, tl = lane % TEAM;
-    const int64_t w0 = (int64_t)blockIdx.x * GC;
-    const int64_t w = w0 + tc < n ? w0 + tc : n - 1;
-    const BoxDev *const gp = boxes + cbox[w];
-    const double4_32a me = sorted[w];
-    const int self = (int)__double_as_longlong(me.w);
-    const int64_t sbase = (int64_t)self * MAXF, ns = n * (int64_t)MAXF;
-    int np, nt;
+    GeomSmem &T = *reinterpret_cast<GeomSmem *>(dyn_smem + (size_t)wid * CPW * sizeof(CellSmem));
     {
-        const unsigned *const row = reinterpret_cast<const unsigned *>(sl.area + sbase);
-        const unsigned h = w0 + tc < n ? row[0] : 0u;
-        np = (int)(h & 255u);
-        nt = (int)(h >> 8);
-        unsigned lv = 0;
-#pragma unroll 2
-        for (int p = tl; p < np; p += TEAM) S.ref[tc][p] = row[1 + p];
-#pragma unroll 2
-        for (int t = tl; 2 * t < nt; t += TEAM) {
-            const unsigned v = row[REC_TRI + t], hi = v >> 16;
-            *reinterpret_cast<unsigned *>(&S.tri[tc][2 * t]) = v;
-            lv |= (1u << (v & 31u)) | (1u << ((v >> 5) & 31u)) | (1u << ((v >> 10) & 31u));
-            if (2 * t + 1 < nt) lv |= (1u << (hi & 31u)) | (1u << ((hi >> 5) & 31u)) | (1u << (hi >> 10));
+        constexpr int NP = CPM / G, NV = CTM / G;
+        unsigned ref[NP], tri[NV], lv = 0;
+        const double off0 = S.off[gl], off8 = S.off[8];
+#pragma unroll
+        for (int r = 0; r < NP; ++r) ref[r] = S.pid[r * G + gl];
+#pragma unroll
+        for (int r = 0; r < NV; ++r) {
+            const unsigned v = tri_of(S.tf[r * G + gl].w);
+            tri[r] = v;
+            if (r * G + gl < nt) lv |= (1u << (v & 31u)) | (1u << ((v >> 5) & 31u)) | (1u << (v >> 10));
         }
 #pragma unroll
-        for (int o = TEAM / 2; o >= 1; o >>= 1) lv |= __shfl_xor_sync(FULL, lv, o);
-        if (tl == 0) {
-            S.live[tc] = lv;
-            S.bad[tc] = 0;
-        }
-        if (tl < 3) {
-            const double p = tl == 0 ? me.x : (tl == 1 ? me.y : me.z), L = gp->L[tl];
-            S.off[tc][3 * tl] = -L - p;
-            S.off[tc][3 * tl + 1] = -p;
-            S.off[tc][3 * tl + 2] = L - p;
+        for (int o = G / 2; o >= 1; o >>= 1) lv |= __shfl_xor_sync(FULL, lv, o);
+        __syncwarp();
+        const int c = gsh / G;
+        T.off[c][gl] = off0;
+#pragma unroll
+        for (int r = 0; r < NP; ++r) T.ref[c][r * G + gl] = ref[r];
+#pragma unroll
+        for (int r = 0; r < NV; ++r) T.tri[c][r * G + gl] = (unsigned short)tri[r];
+        if (gl == 0) {
+            T.off[c][8] = off8;
+            T.live[c] = lv;
+            T.bad[c] = 0;
         }
         __syncwarp();
     }
-    bool todo = nt > 0;
-    while (__any_sync(FULL, todo)) {
-        // ---- the cells of this pass: as many, in order, as the lists hold
-        const int nl = __popc(S.live[tc]);
-        int vb = todo && tl == 0 ? nt : 0, pb = todo && tl == 0 ? nl : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(FULL, vb, o), p = __shfl_up_sync(FULL, pb, o);
-            if (lane >= o) { vb += v; pb += p; }
-        }
-        const bool mine = todo && vb <= GV && pb <= GP;  // prefix sums: true for a first run of the cells left
-        const int nv = __reduce_max_sync(FULL, mine ? vb : 0), npl = __reduce_max_sync(FULL, mine ? pb : 0);
-        vb -= nt;
-        pb -= nl;
-        if (mine && tl == 0) { S.vbase[tc] = vb; S.pbase[tc] = pb; }
-        if (mine) {
-            const unsigned lv = S.live[tc];
-#pragma unroll 1
-            for (unsigned r = lv; r; r &= r - 1u) {
-                const int p = __ffs((int)r) - 1, k = pb + __popc(lv & ((1u << p) - 1u));
-                if ((k & (TEAM - 1)) == tl) S.item[k] = (unsigned short)(tc << 5 | p);
-            }
-#pragma unroll 2
-            for (int t = tl; t < nt; t += TEAM) S.vitem[vb + t] = (unsigned short)(tc << 6 | t);
-        }
-        if (lane < 16) S.hist[lane] = 0;
-        {
-            uint4 *const z = reinterpret_cast<uint4 *>(&S.nxt[0][0]);
-#pragma unroll 2
-            for (int i = lane; i < npl * CPM / 16; i += 32) z[i] = make_uint4(FULL, FULL, FULL, FULL);
-        }
-        __syncwarp();
-        // ---- planes and edges
-#pragma unroll 1
-        for (int k = lane; k < npl; k += 32) {
-            const int it = S.item[k], c = it >> 5;
-            double x, y, z, o;
-            const int64_t wc = w0 + c;
-            plane64(S.off[c], S.ref[c][it & 31], sorted, boxes + cbox[wc], x, y, z, o);
-            S.px[k] = x; S.py[k] = y; S.pz[k] = z; S.po[k] = o;
-            S.vp[k] = 0.0;
-        }
-#pragma unroll 1
-        for (int k = lane; k < nv; k += 32) {
-            const int it = S.vitem[k], c = it >> 6, t = it & 63;
-            const unsigned v = S.tri[c][t], x = v & 31u, y = (v >> 5) & 31u, z = v >> 10;
-            S.nxt[plane_of(S, c, x)][y] = (unsigned char)t;
-            S.nxt[plane_of(S, c, y)][z] = (unsigned char)t;
-            S.nxt[plane_of(S, c, z)][x] = (unsigned char)t;
-        }
-        __syncwarp();
-        // ---- vertices; an edge two triangles claim is not a closed cell
-#pragma unroll 1
-        for (int k = lane; k < nv; k += 32) {
-            const int it = S.vitem[k], c = it >> 6, t = it & 63;
-            const unsigned v = S.tri[c][t], x = v & 31u, y = (v >> 5) & 31u, z = v >> 10;
-            const int a = plane_of(S, c, x), b = plane_of(S, c, y), d = plane_of(S, c, z);
-            if (S.nxt[a][y] != t || S.nxt[b][z] != t || S.nxt[d][x] != t) S.bad[c] = 1;
-            vertex64(S, a, b, d, S.vx[k], S.vy[k], S.vz[k]);
-        }
-        // ---- faces by number of vertices: the bytes of the edge row in use
-#pragma unroll 1
-        for (int k = lane; k < npl; k += 32) {
-            const uint4 *const r = reinterpret_cast<const uint4 *>(S.nxt[k]);
-            const uint4 a = r[0], b = r[1];
-            const unsigned u = ~a.x & 0x80808080u, v = ~a.y & 0x80808080u, x = ~a.z & 0x80808080u, y = ~a.w & 0x80808080u;
-            const unsigned u2 = ~b.x & 0x80808080u, v2 = ~b.y & 0x80808080u, x2 = ~b.z & 0x80808080u, y2 = ~b.w & 0x80808080u;
-            const int d = min(__popc(u | v >> 1 | x >> 2 | y >> 3 | u2 >> 4 | v2 >> 5 | x2 >> 6 | y2 >> 7), 15);
-            S.deg[k] = (unsigned char)d;
-            atomicAdd(&S.hist[d], 1);
-        }
-        __syncwarp();
-        {
-            const int h = lane < 16 ? S.hist[15 - lane] : 0;  // most vertices first
-            int p = h;
-#pragma unroll
-            for (int o = 1; o < 16; o <<= 1) {
-                const int q = __shfl_up_sync(FULL, p, o);
-                if (lane >= o) p += q;
-            }
-            if (lane < 16) S.hist[15 - lane] = p - h;
-        }
-        __syncwarp();
-#pragma unroll 1
-        for (int k = lane; k < npl; k += 32) S.order[atomicAdd(&S.hist[S.deg[k]], 1)] = (unsigned short)k;
-        __syncwarp();
-#pragma unroll 1
-        for (int j = lane; j < npl; j += 32) {
-            const int k = S.order[j], it = S.item[k], c = it >> 5;
-            const unsigned p = it & 31;
-            const int vbc = S.vbase[c];
-            // the walk starts at the vertex holding the edge to the lowest slot
-            unsigned y = 0;
-            int t0 = 255;
-            {
-                const uint4 *const r = reinterpret_cast<const uint4 *>(S.nxt[k]);
-                const uint4 a = r[0], b = r[1];
-                const unsigned wv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-                for (int q = 7; q >= 0; --q) {
-                    const unsigned u = ~wv[q] & 0x80808080u;
-                    if (u) {
-                        const int s = __ffs((int)u) >> 3;  // byte 0..3 (its bit 7 is set)
-                        y = (unsigned)(4 * q + s - 1);
-                        t0 = (int)((wv[q] >> (8 * (s - 1))) & 255u);
-                    }
-                }
-            }
-            const double qx = S.px[k], qy = S.py[k], qz = S.pz[k];
-            const int ka = fan_axis(qx, qy, qz);
-            const double *T1 = (ka == 0 ? S.vy : S.vx) + vbc, *T2 = (ka == 2 ? S.vy : S.vz) + vbc;
-            const double u0 = T1[t0], v0 = T2[t0];
-            FaceFan F;
-            bool ok = false, any = false;
-#pragma unroll 1
-            for (int guard = 0; guard < CTM; ++guard) {
-                const unsigned vt = S.tri[c][guard == 0 ? t0 : (int)S.nxt[k][y]];
-                y = (vt & 31u) ^ ((vt >> 5) & 31u) ^ (vt >> 10) ^ p ^ y;
-                const int tn = S.nxt[k][y];
-                if (tn == 255) break;
-                if (tn == t0) { ok = true; break; }
-                const double bu = T1[tn] - u0, bv = T2[tn] - v0;
-                if (any) F.edge(bu, bv);
-                else F.begin(bu, bv);
-                any = true;
-            }
-            if (!ok) S.bad[c] = 1;
-            double area, fx, fy, fz, vp;
-            face_of_fan(F, ka, qx, qy, qz, S.po[k], S.vx[vbc + t0], S.vy[vbc + t0], S.vz[vbc + t0], area, fx, fy, fz, vp);
-            S.px[k] = area; S.py[k] = fx; S.pz[k] = fy; S.po[k] = fz;
-            S.vp[k] = vp;
-        }
-        __syncwarp();
-        // ---- slots, cell by cell in order of the planes
-        const double amin = gp->amin;
-        int nface = 0;
-        {
-            const int nout = mine && !S.bad[tc] ? nl : 0, maxout = __reduce_max_sync(FULL, nout);
-#pragma unroll 1
-            for (int i = tl; i - tl < maxout; i += TEAM) {
-                const int k = pb + i;
-                const bool keep = i < nout && abs_bits(S.px[k]) > abs_bits(amin);
-                const unsigned km = (__ballot_sync(FULL, keep) >> (tc * TEAM)) & ((1u << TEAM) - 1u);
-                if (keep) {
-                    const int64_t s = sbase + nface + __popc(km & ((1u << tl) - 1u));
-                    const unsigned ref = S.ref[tc][S.item[k] & 31], code = ref >> 27;
-                    int nb = self, sh;
-                    if (code == 31u) {
-                        const int kf = (int)(ref & 7u), d = kf >> 1, e = d == 0 ? 1 : (d == 1 ? 3 : 9);
-                        sh = 13 + ((kf & 1) ? -e : e);
-                    } else {
-                        nb = (int)__double_as_longlong(sorted[ref & IDX_MASK].w);
-                        sh = (int)code;
-                    }
-                    sl.nb[s] = nb;
-                    sl.sh[s] = (unsigned char)sh;
-                    sl.area[s] = S.px[k];
-                    sl.fc[s] = S.py[k];
-                    sl.fc[ns + s] = S.pz[k];
-                    sl.fc[2 * ns + s] = S.po[k];
-                }
-                nface += __popc(km);
-            }
-        }
-        __syncwarp();
-        // ---- volume and first moment: k_clip's tree over the 32 slots (p and
-        // p + 16, then p + 8, p + 4, p + 2, p + 1; a slot without a face adds 0)
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        {
-            const unsigned lv = S.live[tc];
-            double b[4][4];
-            // lane tl sums slots tl + {0, 16, 8, 24, 4, 20, 12, 28}
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                for (int g = 0; g < 2; ++g) {
-                    double s[2][4];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int p = tl + 4 * h + 8 * g + 16 * e;
-                        const bool has = mine && ((lv >> p) & 1u);
-                        const int k = has ? pb + __popc(lv & ((1u << p) - 1u)) : 0;
-                        const double vp = has ? S.vp[k] : 0.0, vw = 0.75 * vp;
-                        s[e][0] = vp;
-                        s[e][1] = has ? __dmul_rn(vw, S.py[k]) : 0.0;
-                        s[e][2] = has ? __dmul_rn(vw, S.pz[k]) : 0.0;
-                        s[e][3] = has ? __dmul_rn(vw, S.po[k]) : 0.0;
-                    }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) b[2 * h + g][q] = __dadd_rn(s[0][q], s[1][q]);
-                }
-            }
-            a0 = __dadd_rn(__dadd_rn(b[0][0], b[1][0]), __dadd_rn(b[2][0], b[3][0]));
-            a1 = __dadd_rn(__dadd_rn(b[0][1], b[1][1]), __dadd_rn(b[2][1], b[3][1]));
-            a2 = __dadd_rn(__dadd_rn(b[0][2], b[1][2]), __dadd_rn(b[2][2], b[3][2]));
-            a3 = __dadd_rn(__dadd_rn(b[0][3], b[1][3]), __dadd_rn(b[2][3], b[3][3]));
-        }
-#pragma unroll
-        for (int o = TEAM / 2; o >= 1; o >>= 1) {
-            a0 += __shfl_xor_sync(FULL, a0, o);
-            a1 += __shfl_xor_sync(FULL, a1, o);
-            a2 += __shfl_xor_sync(FULL, a2, o);
-            a3 += __shfl_xor_sync(FULL, a3, o);
-        }
-        if (mine && tl == 0) {
-            if (S.bad[tc]) {
-                list[atomicAdd(list_n, 1)] = (int)w;
-            } else {
-                sl.cnt[self] = nface;
-                vol[self] = a0;
-                cen[self] = a1;
-                cen[n + self] = a2;
-                cen[2 * n + self] = a3;
-            }
-        }
-        todo = todo && !mine;
-        __syncwarp();
-    }
+    warp_geometry(T, lane, w0, w, nt, gp, self, sorted, n, boxes, cbox, vol, cen, sl, list, list_n);
 }
 
 }  // namespace
@@ -1055,12 +1048,10 @@ void launch_cells(const double4_32a *sorted, const float4 *sortedf, const int *s
 {
     constexpr int WARPS = 2, CELLS = WARPS * 32 / LANES;
     constexpr size_t smem = sizeof(CellSmem) * CELLS;
-    static_assert(smem <= 48 * 1024 && sizeof(GeomSmem) <= 48 * 1024, "no opt-in needed");
+    static_assert(smem <= 48 * 1024, "no opt-in needed");
     cand_cap = cand_cap < 32 ? 32 : (cand_cap > CCB ? CCB : cand_cap);
     k_cells<LANES><<<(unsigned)((n + CELLS - 1) / CELLS), 32 * WARPS, smem, s>>>(sorted, sortedf, start, n, boxes, cbox,
-                                                                                sl, cand_cap, list, list_n);
-    k_cell_geom<<<(unsigned)((n + GC - 1) / GC), 32, sizeof(GeomSmem), s>>>(sorted, n, boxes, cbox, vol, cen, sl, list,
-                                                                         list_n);
+                                                                                vol, cen, sl, cand_cap, list, list_n);
 }
 
 }  // namespace mm

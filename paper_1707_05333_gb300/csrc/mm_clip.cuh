@@ -3,6 +3,7 @@
 // their error bounds.
 #pragma once
 
+#include "mm_fp64.cuh"
 #include "mm_internal.cuh"
 
 namespace mm {
@@ -29,22 +30,20 @@ __device__ __forceinline__ long long abs_bits(double x)
 }
 // Intersection of planes a, b, c in FP64 with explicitly rounded operations
 // (so every caller gets the same bits):
-// x = (o_a (q_b x q_c) + o_b (q_c x q_a) + o_c (q_a x q_b)) / det(q_a, q_b, q_c).
+// x = (o_a (q_b x q_c) + q_a x (o_c q_b - o_b q_c)) / det(q_a, q_b, q_c),
+// 30 FP64 operations (Cramer's rule with all three cross products: 36).
 __device__ __forceinline__ void solve64(double ax, double ay, double az, double ao, double bx, double by, double bz,
                                         double bo, double cx, double cy, double cz, double co, double &x, double &y,
                                         double &z)
 {
-    const double bcx = __fma_rn(by, cz, -__dmul_rn(bz, cy)), bcy = __fma_rn(bz, cx, -__dmul_rn(bx, cz)),
-                 bcz = __fma_rn(bx, cy, -__dmul_rn(by, cx));
-    const double cax = __fma_rn(cy, az, -__dmul_rn(cz, ay)), cay = __fma_rn(cz, ax, -__dmul_rn(cx, az)),
-                 caz = __fma_rn(cx, ay, -__dmul_rn(cy, ax));
-    const double abx = __fma_rn(ay, bz, -__dmul_rn(az, by)), aby = __fma_rn(az, bx, -__dmul_rn(ax, bz)),
-                 abz = __fma_rn(ax, by, -__dmul_rn(ay, bx));
-    const double det = __fma_rn(ax, bcx, __fma_rn(ay, bcy, __dmul_rn(az, bcz)));
-    const double inv = __drcp_rn(det);
-    x = __dmul_rn(__fma_rn(ao, bcx, __fma_rn(bo, cax, __dmul_rn(co, abx))), inv);
-    y = __dmul_rn(__fma_rn(ao, bcy, __fma_rn(bo, cay, __dmul_rn(co, aby))), inv);
-    z = __dmul_rn(__fma_rn(ao, bcz, __fma_rn(bo, caz, __dmul_rn(co, abz))), inv);
+    const double nx = __fma_rn(by, cz, -__dmul_rn(bz, cy)), ny = __fma_rn(bz, cx, -__dmul_rn(bx, cz)),
+                 nz = __fma_rn(bx, cy, -__dmul_rn(by, cx));
+    const double dx = __fma_rn(co, bx, -__dmul_rn(bo, cx)), dy = __fma_rn(co, by, -__dmul_rn(bo, cy)),
+                 dz = __fma_rn(co, bz, -__dmul_rn(bo, cz));
+    const double inv = rcp64(__fma_rn(ax, nx, __fma_rn(ay, ny, __dmul_rn(az, nz))));
+    x = __dmul_rn(__fma_rn(ao, nx, __fma_rn(ay, dz, -__dmul_rn(az, dy))), inv);
+    y = __dmul_rn(__fma_rn(ao, ny, __fma_rn(az, dx, -__dmul_rn(ax, dz))), inv);
+    z = __dmul_rn(__fma_rn(ao, nz, __fma_rn(ax, dy, -__dmul_rn(ay, dx))), inv);
 }
 template <class S_t>
 __device__ __forceinline__ void vertex64(const S_t &S, int a, int b, int c, double &x, double &y, double &z)
@@ -152,22 +151,21 @@ __device__ __forceinline__ void face_of_fan(const FaceFan &F, int k, double qx, 
 {
     const double qk = k == 0 ? qx : (k == 1 ? qy : qz);
     const double q1 = k == 0 ? qy : qx, q2 = k == 2 ? qy : qz;
-    const double aw = fabs(F.W);
-    const double qn2 = __dmul_rn(2.0, o);  // |q|^2
     // 1 / q_k and 1 / (3 W) from one reciprocal of 3 W q_k; a face
     // of zero fan weight (area 0) takes 0 for both
     const double w3 = __dmul_rn(3.0, F.W);
     const bool nz = abs_bits(F.W) != 0;
-    const double r = nz ? 1.0 / __dmul_rn(w3, qk) : 0.0;
-    const double iq = __dmul_rn(w3, r), iqk = fabs(iq);
-    area = __dmul_rn(__dmul_rn(__dmul_rn(0.5, aw), __dmul_rn(qn2, rsqrt(qn2))), iqk);
+    const double r = nz ? rcp64(__dmul_rn(w3, qk)) : 0.0;
+    const double iq = __dmul_rn(w3, r);
+    const double s = fabs(__dmul_rn(F.W, iq));            // |W / q_k|
+    area = __dmul_rn(s, __dmul_rn(o, rsqrt64(2.0 * o)));  // o / |q| = |q| / 2
+    vp = __dmul_rn(s, __dmul_rn(o, 1.0 / 6.0));           // |q|^2 / 12
     const double i3w = __dmul_rn(qk, r);
     const double du = __dmul_rn(F.su, i3w), dv = __dmul_rn(F.sv, i3w);
     const double dk = __dmul_rn(-__fma_rn(q1, du, __dmul_rn(q2, dv)), iq);
     fx = __dadd_rn(x0, k == 0 ? dk : du);
     fy = __dadd_rn(y0, k == 1 ? dk : (k == 0 ? du : dv));
     fz = __dadd_rn(z0, k == 2 ? dk : dv);
-    vp = __dmul_rn(__dmul_rn(__dmul_rn(aw, qn2), iqk), 1.0 / 12.0);
 }
 
 }  // namespace mm

@@ -1,0 +1,46 @@
+// mm_fp64.cuh -- FP64 reciprocal, quotient and reciprocal square root by one
+// third-order iteration.
+//
+// GB300 issues an FP64 instruction in 16 cycles of the SM's pipe, so their
+// number is what the kernels with FP64 arithmetic cost.  The hardware's seed
+// (rcp/rsqrt.approx.ftz.f64, about 20 good bits) with residual e = 1 - x y
+// gives 1/x = y / (1 - e) = y (1 + e + e^2) + O(e^3): 2^-60 relative, then one
+// rounding, in three instructions.  Outside 2^+-1000 the seed would flush and
+// the library operation is taken.
+#pragma once
+
+namespace mm {
+
+__device__ __forceinline__ bool seed_range(double x)
+{
+    return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 23u < 2000u;
+}
+
+__device__ __forceinline__ double rcp64(double x)
+{
+    if (!seed_range(x)) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = __fma_rn(-x, y, 1.0);
+    return __fma_rn(y, __fma_rn(e, e, e), y);
+}
+
+// a / b with the quotient's own residual folded back in
+__device__ __forceinline__ double div64(double a, double b)
+{
+    const double y = rcp64(b), q = __dmul_rn(a, y);
+    const double r = __fma_rn(__fma_rn(-b, q, a), y, q);
+    return seed_range(q) ? r : a / b;  // a quotient near the range's ends, or 0: the library's
+}
+
+// 1 / sqrt(x), x > 0: with e = 1 - x y^2, y (1 + e/2 + 3 e^2 / 8)
+__device__ __forceinline__ double rsqrt64(double x)
+{
+    if (!seed_range(x)) return rsqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    return __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
+}
+
+}  // namespace mm
