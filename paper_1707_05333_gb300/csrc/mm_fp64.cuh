@@ -30,7 +30,8 @@ __device__ __forceinline__ double div64(double a, double b)
 {
     const double y = rcp64(b), q = __dmul_rn(a, y);
     const double r = __fma_rn(__fma_rn(-b, q, a), y, q);
-    return seed_range(q) ? r : a / b;  // a quotient near the range's ends, or 0: the library's
+    // a quotient near the range's ends (zero is exact): the library's
+    return seed_range(q) || (__double_as_longlong(q) << 1) == 0 ? r : a / b;
 }
 
 // 1 / sqrt(x), x > 0: with e = 1 - x y^2, y (1 + e/2 + 3 e^2 / 8)

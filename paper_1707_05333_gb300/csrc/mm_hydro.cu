@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(128, MM_GRAD_MINBLOCKS) k_gradient(MeshDev m, 
         const double c00 = M[4] * M[8] - M[5] * M[7], c01 = M[5] * M[6] - M[3] * M[8], c02 = M[3] * M[7] - M[4] * M[6];
         const double c10 = M[2] * M[7] - M[1] * M[8], c11 = M[0] * M[8] - M[2] * M[6], c12 = M[1] * M[6] - M[0] * M[7];
         const double c20 = M[1] * M[5] - M[2] * M[4], c21 = M[2] * M[3] - M[0] * M[5], c22 = M[0] * M[4] - M[1] * M[3];
-        const double idet = 1.0 / (M[0] * c00 + M[1] * c01 + M[2] * c02);
+        const double idet = rcp64(M[0] * c00 + M[1] * c01 + M[2] * c02);
         mi[0] = c00 * idet; mi[1] = c10 * idet; mi[2] = c20 * idet;
         mi[3] = c01 * idet; mi[4] = c11 * idet; mi[5] = c21 * idet;
         mi[6] = c02 * idet; mi[7] = c12 * idet; mi[8] = c22 * idet;
@@ -273,13 +273,27 @@ __global__ void __launch_bounds__(128, MM_GRAD_MINBLOCKS) k_gradient(MeshDev m, 
         double al[NG];
 #pragma unroll
         for (int k = 0; k < NG; ++k) {
-            // the ratios matter only below 1 (min(1, x)), so most cells skip the
-            // FP64 divisions: x < 1 exactly when the numerator is the smaller
+            // min(1, up / dmax, dn / dmin): the ratios matter only below 1, which
+            // is where the numerator is the smaller in magnitude, and of two
+            // ratios the products tell the smaller, so that a column takes one
+            // FP64 division at most (six instructions; a product is one): the two
+            // passes of the 256^3 shear layer 30.3 + 21.4 -> 28.6 + 19.6 ms
             double a = 1.0;
-            const double up = okey_value(kx[k]) - Wi[k], dn = okey_value(kn[k]) - Wi[k];
-            const double dmax = okey_value(kdx[k]), dmin = okey_value(kdn[k]);
-            if (kdx[k] > 0 && up < dmax) a = fmin(a, up / dmax);
-            if (kdn[k] < 0 && dn > dmin) a = fmin(a, dn / dmin);
+            double up = okey_value(kx[k]) - Wi[k], dmax = okey_value(kdx[k]);
+            const double dn = okey_value(kn[k]) - Wi[k], dmin = okey_value(kdn[k]);
+            // (okey(-0) is -1: a minimum below zero is below that)
+            const bool over = kdx[k] > 0 && okey(up) < kdx[k], under = kdn[k] < -1 && okey(dn) > kdn[k];
+            if (over || under) {
+                bool second = !over;
+                if (over && under) {
+                    const double u = up * dmin, d = dn * dmax;  // both below 0 or zero
+                    second = okey(d) > okey(u);
+                    // (products out of range tell nothing: both quotients)
+                    if (!seed_range(u) || !seed_range(d)) second = dn / dmin < up / dmax;
+                }
+                if (second) { up = dn; dmax = dmin; }
+                a = div64(up, dmax);
+            }
             al[k] = a;
         }
         if (c.limiter == 2) {
@@ -334,7 +348,7 @@ __global__ void __launch_bounds__(128, MM_GRAD_MINBLOCKS) k_gradient(MeshDev m, 
     // (rho, m, E):  d_d u_k = (d_d m_k - u_k d_d rho) / rho,
     // d_d P = (gamma-1)(d_d E - u . d_d m + |u|^2/2 d_d rho)
     const double gm1 = c.gamma - 1.0;
-    const double ir = 1.0 / Wi[0];
+    const double ir = rcp64(Wi[0]);
     const double ux = Wi[1] * ir, uy = Wi[2] * ir, uz = Wi[3] * ir;
     const double u2 = ux * ux + uy * uy + uz * uz;
     const double P = gm1 * (Wi[4] - 0.5 * Wi[0] * u2);
@@ -397,6 +411,10 @@ void launch_gradient(const MeshDev &m, const HydroCfg &c, const double *W, const
 // ---------------------------------------------------------------------------
 using FaceState = FaceStateT<double>;
 
+// Bound by the FP64 pipe (90 % busy at 234 instructions a face): the count is
+// the cost.  Reciprocals of mm_fp64.cuh, two operations a momentum component
+// (hllc_t), floors compared as integers and no offsets added to faces inside
+// the box: 54.2 -> 47.5 ms for the 133 million faces of the 256^3 shear layer.
 // With NG = 6 the flux rows 5, 6 and 7 hold the entropy flux A F_(rho A), the
 // face's shock Mach number and its swept-volume rate A (w_f . n).
 template <int NG>
@@ -409,21 +427,29 @@ __global__ void __launch_bounds__(128) k_face_flux(MeshDev m, HydroCfg c, const 
     const int64_t n = m.n, fs = m.fs;
     const int i = m.face_i[f], j = m.face_j[f];
     const int code = m.face_shift[f];
-    const double *Lb = m.boxL + 3 * m.cbox[i];
-    const double ox = image_axis(code % 3, Lb[0]), oy = image_axis((code / 3) % 3, Lb[1]),
-                 oz = image_axis(code / 9, Lb[2]);
+    // side j's generator and centroid in side i's frame (faces inside the box
+    // add no offset)
+    double rjx = pos[j], rjy = pos[n + j], rjz = pos[2 * n + j];
+    double cjx = m.cen[j], cjy = m.cen[n + j], cjz = m.cen[2 * n + j];
+    if (code != 13) {
+        const double *Lb = m.boxL + 3 * m.cbox[i];
+        const double ox = image_axis(code % 3, Lb[0]), oy = image_axis((code / 3) % 3, Lb[1]),
+                     oz = image_axis(code / 9, Lb[2]);
+        rjx += ox; rjy += oy; rjz += oz;
+        cjx += ox; cjy += oy; cjz += oz;
+    }
     const double fx = m.fcen[f], fy = m.fcen[fs + f], fz = m.fcen[2 * fs + f];
     const double nx = m.normal[f], ny = m.normal[fs + f], nz = m.normal[2 * fs + f];
     // reconstruction to the face centroid: W_face = W_half + (x_f - c) . grad
     const double dlx = fx - m.cen[i], dly = fy - m.cen[n + i], dlz = fz - m.cen[2 * n + i];
-    const double drx = fx - (m.cen[j] + ox), dry = fy - (m.cen[n + j] + oy), drz = fz - (m.cen[2 * n + j] + oz);
+    const double drx = fx - cjx, dry = fy - cjy, drz = fz - cjz;
     double WL[NG], WR[NG];
 #pragma unroll
     for (int k = 0; k < NG; ++k) {
         WL[k] = Wh[k * n + i] + dlx * grad[(3 * k) * n + i] + dly * grad[(3 * k + 1) * n + i] + dlz * grad[(3 * k + 2) * n + i];
         WR[k] = Wh[k * n + j] + drx * grad[(3 * k) * n + j] + dry * grad[(3 * k + 1) * n + j] + drz * grad[(3 * k + 2) * n + j];
     }
-    const bool vac_l = !(WL[0] >= c.rho_floor), vac_r = !(WR[0] >= c.rho_floor);
+    const bool vac_l = NG == 6 && !(WL[0] >= c.rho_floor), vac_r = NG == 6 && !(WR[0] >= c.rho_floor);
     double irl, irr, kel, ker;
     apply_floor_ir_t<double>(WL, c.rho_floor, c.eps_floor, irl, kel);
     apply_floor_ir_t<double>(WR, c.rho_floor, c.eps_floor, irr, ker);
@@ -436,11 +462,10 @@ __global__ void __launch_bounds__(128) k_face_flux(MeshDev m, HydroCfg c, const 
     // face velocity (Sec. 4): mean generator velocity plus the correction for
     // the face centroid lying off the generators' midpoint
     const double rix = pos[i], riy = pos[n + i], riz = pos[2 * n + i];
-    const double rjx = pos[j] + ox, rjy = pos[n + j] + oy, rjz = pos[2 * n + j] + oz;
     const double drgx = rjx - rix, drgy = rjy - riy, drgz = rjz - riz;
     const double wix = w[i], wiy = w[n + i], wiz = w[2 * n + i];
     const double wjx = w[j], wjy = w[n + j], wjz = w[2 * n + j];
-    const double il2 = 1.0 / (drgx * drgx + drgy * drgy + drgz * drgz);
+    const double il2 = rcp64(drgx * drgx + drgy * drgy + drgz * drgz);
     const double corr = ((wix - wjx) * (fx - 0.5 * (rix + rjx)) + (wiy - wjy) * (fy - 0.5 * (riy + rjy)) +
                          (wiz - wjz) * (fz - 0.5 * (riz + rjz))) * il2;
     const double wfx = corr * drgx + 0.5 * (wix + wjx);

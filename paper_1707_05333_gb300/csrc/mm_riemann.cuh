@@ -2,6 +2,8 @@
 // FP64 and the mixed-precision hydro kernels (Sec. 4, Sec. 4.1).
 #pragma once
 
+#include "mm_fp64.cuh"
+
 namespace mm {
 
 // Wave speeds of a face's Riemann problem along the unit normal, for the
@@ -32,6 +34,18 @@ __device__ __forceinline__ double okey_value(long long k)
     return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
 }
 
+// 1 / x and a / b: in FP64 by the short sequences of mm_fp64.cuh
+__device__ __forceinline__ double inv_t(double x) { return rcp64(x); }
+__device__ __forceinline__ float inv_t(float x) { return 1.0f / x; }
+__device__ __forceinline__ double quot_t(double a, double b) { return div64(a, b); }
+__device__ __forceinline__ float quot_t(float a, float b) { return a / b; }
+// a >= b: FP64 by integers (false where either is NaN, as the operator)
+__device__ __forceinline__ bool not_below_t(double a, double b)
+{
+    const long long inf = 0x7ff0000000000000LL;
+    return okey(a) >= okey(b) && okey(a) <= inf;
+}
+__device__ __forceinline__ bool not_below_t(float a, float b) { return a >= b; }
 __device__ __forceinline__ double sqrt_t(double x) { return sqrt(x); }
 __device__ __forceinline__ float sqrt_t(float x) { return sqrtf(x); }
 __device__ __forceinline__ double min_t(double a, double b) { return okey(a) < okey(b) ? a : b; }
@@ -65,7 +79,7 @@ __device__ __forceinline__ void hllc_t(const FaceStateT<T> &L, const FaceStateT<
     const T sl = min_t(ul - cl, ur - cr);
     const T sr = max_t(ul + cl, ur + cr);
     const T ml = L.rho * (sl - ul), mr = R.rho * (sr - ur);
-    const T ss = (R.P - L.P + ul * ml - ur * mr) / (ml - mr);
+    const T ss = quot_t(R.P - L.P + ul * ml - ur * mr, ml - mr);
     if (wv) *wv = WavesT<T>{sl, sr, ss, ul, ur};
     const bool left = nonneg_t(sl) || nonneg_t(ss);
     const bool star = !nonneg_t(sl) && (left || pos_t(sr));
@@ -73,29 +87,29 @@ __device__ __forceinline__ void hllc_t(const FaceStateT<T> &L, const FaceStateT<
     const T uk = left ? ul : ur;
     const T Ek = left ? El : Er;
     const T sk = left ? sl : sr;
-    const T mk = K.rho * uk;
-    // physical flux of side K
-    F[0] = mk;
-    F[1] = mk * K.vx + K.P * nx;
-    F[2] = mk * K.vy + K.P * ny;
-    F[3] = mk * K.vz + K.P * nz;
+    // Flux of side K, F_K, or across the star state, F_K + S_K (U*_K - U_K) with
+    // U*_K = rho_K (S_K - u_K)/(S_K - S*) (1, v_K + (S* - u_K) n, E_K/rho_K + (S* - u_K)(S* + P_K/(rho_K (S_K - u_K)))).
+    // Both have the momentum flux F_0 v_K + p n: F_0 the mass flux, p = P_K or
+    // P_K + S_K f (S* - u_K), so a component costs two operations.
+    F[0] = K.rho * uk;
+    T p = K.P;
     F[4] = (Ek + K.P) * uk;
     if (star) {
-        // U*_K = rho_K (S_K - u_K)/(S_K - S*) (1, v_K + (S* - u_K) n, E_K/rho_K + (S* - u_K)(S* + P_K/(rho_K (S_K - u_K))))
         // With f = rho_K (S_K - u_K) / (S_K - S*), the energy term
         // f (S* - u_K) P_K / (rho_K (S_K - u_K)) equals (S* - u_K) P_K / (S_K - S*):
         // written that way the star state needs one division, and stays finite
         // where S_K rounds to u_K (a sound speed below the flow speed's ulp).
-        const T rb = T(1) / (sk - ss);
+        const T rb = inv_t(sk - ss);
         const T f = K.rho * (sk - uk) * rb;
         const T du = ss - uk;
         const T es = f * (Ek * K.irho + du * ss) + du * K.P * rb;
         F[0] += sk * (f - K.rho);
-        F[1] += sk * (f * (K.vx + du * nx) - K.rho * K.vx);
-        F[2] += sk * (f * (K.vy + du * ny) - K.rho * K.vy);
-        F[3] += sk * (f * (K.vz + du * nz) - K.rho * K.vz);
+        p += sk * (f * du);
         F[4] += sk * (es - Ek);
     }
+    F[1] = F[0] * K.vx + p * nx;
+    F[2] = F[0] * K.vy + p * ny;
+    F[3] = F[0] * K.vz + p * nz;
 }
 
 // HLL with the same wave speeds: one intermediate state from the integral
@@ -184,7 +198,7 @@ __device__ __forceinline__ void riemann_t(int kind, const FaceStateT<T> &L, cons
 template <class T>
 __device__ __forceinline__ void apply_floor_ir_t(T W[5], T rho_floor, T eps_floor, T &ir, T &ke)
 {
-    if (!(W[0] >= rho_floor)) {
+    if (!not_below_t(W[0], rho_floor)) {
         W[0] = rho_floor;
         W[1] = W[2] = W[3] = T(0);
         W[4] = rho_floor * eps_floor;
@@ -192,9 +206,9 @@ __device__ __forceinline__ void apply_floor_ir_t(T W[5], T rho_floor, T eps_floo
         ke = T(0);
         return;
     }
-    ir = T(1) / W[0];
+    ir = inv_t(W[0]);
     ke = T(0.5) * (W[1] * W[1] + W[2] * W[2] + W[3] * W[3]) * ir;
-    if (!(W[4] - ke >= W[0] * eps_floor)) W[4] = W[0] * eps_floor + ke;
+    if (!not_below_t(W[4] - ke, W[0] * eps_floor)) W[4] = W[0] * eps_floor + ke;
 }
 
 // Floors on density and specific internal energy (Sec. 4.1).  A state below
