@@ -87,6 +87,27 @@ __device__ __forceinline__ void hllc_t(const FaceStateT<T> &L, const FaceStateT<
     const T uk = left ? ul : ur;
     const T Ek = left ? El : Er;
     const T sk = left ? sl : sr;
+    if constexpr (sizeof(T) == 4) {
+        // FP32: the sums component by component (the order its results carry)
+        const T mk = K.rho * uk;
+        F[0] = mk;
+        F[1] = mk * K.vx + K.P * nx;
+        F[2] = mk * K.vy + K.P * ny;
+        F[3] = mk * K.vz + K.P * nz;
+        F[4] = (Ek + K.P) * uk;
+        if (star) {
+            const T rb = T(1) / (sk - ss);
+            const T f = K.rho * (sk - uk) * rb;
+            const T du = ss - uk;
+            const T es = f * (Ek * K.irho + du * ss) + du * K.P * rb;
+            F[0] += sk * (f - K.rho);
+            F[1] += sk * (f * (K.vx + du * nx) - K.rho * K.vx);
+            F[2] += sk * (f * (K.vy + du * ny) - K.rho * K.vy);
+            F[3] += sk * (f * (K.vz + du * nz) - K.rho * K.vz);
+            F[4] += sk * (es - Ek);
+        }
+        return;
+    }
     // Flux of side K, F_K, or across the star state, F_K + S_K (U*_K - U_K) with
     // U*_K = rho_K (S_K - u_K)/(S_K - S*) (1, v_K + (S* - u_K) n, E_K/rho_K + (S* - u_K)(S* + P_K/(rho_K (S_K - u_K)))).
     // Both have the momentum flux F_0 v_K + p n: F_0 the mass flux, p = P_K or
