@@ -10,10 +10,11 @@
 //
 // What bounds it and what it measured (GB300, jittered 64^3 lattice and
 // 200003 random generators, ncu durations; k_clip took 5.89 and 8.89 ms):
-// 2.77 and 4.28 ms, of dependent latencies with 15 warps an SM (3.4 KB of
-// shared memory a cell, 128 registers): 1.6 instructions a cycle, 5340 a cell
-// against k_clip's 14200, and the FP64 pipe 51 % busy with 106 instructions a
-// cell against 236.
+// 2.73 and 4.26 ms, of dependent latencies with 15 warps an SM (3.4 KB of
+// shared memory a cell, 128 registers): 1.6 instructions a cycle, 5220 a cell
+// against k_clip's 14200, and the FP64 pipe 52 % busy with 107 instructions a
+// cell against 236.  (18 warps an SM at 96 registers gained nothing: the
+// misses of the instruction cache doubled.)
 //  * Loops are kept rolled: unrolled, the body outgrew the instruction cache
 //    and half of the cycles went to fetching it (5.3 and 13.0 ms).
 //  * Screening candidates a lane each after the first 16 instead of trying all
@@ -23,7 +24,7 @@
 //    kernel and the issue slots in the other: 3.15 and 4.68 ms in all, here
 //    2.88 and 4.33 before the shorter FP64 sequences (mm_fp64.cuh, solve64).
 //
-// A cell that outgrows these lists (more than 32 live planes, 48 vertices, 32
+// A cell that outgrows these lists (more than 32 live planes, 56 vertices, 32
 // new vertices in a cut, CELL_RINGS search rings), holds a coincident
 // generator or has an inconsistent cut goes to a list that the warp-per-cell
 // clipper works through next, so nothing is refused here.
@@ -34,10 +35,10 @@ namespace mm {
 namespace {
 
 constexpr int CPM = 32;    // live planes: one bit of a word
-constexpr int CTM = 48;    // vertices
+constexpr int CTM = 56;    // vertices
 constexpr int CNS = 32;    // new (and removed) vertices of one cut
 constexpr int CCB = 64;    // candidate buffer, flushed as in k_clip
-constexpr int CELL_RINGS = 4;
+constexpr int CELL_RINGS = 6;
 constexpr int SCREEN = 16;
 constexpr int LANES = 8;   // lanes a cell (16 lanes: jittered 64^3 2.35 ms for 1.70, random generators the same)
 constexpr unsigned BOX_PLANE = 31u << 27;  // plane reference of box face k: BOX_PLANE | k
@@ -45,7 +46,7 @@ constexpr unsigned IDX_MASK = 0x7ffffffu;  // sorted index of a plane reference 
 static_assert(MM_MAX_CELLS < (1LL << 27), "a plane reference holds the index in 27 bits");
 
 struct __align__(16) CellSmem {
-    float4 tf[CTM];       // vertex; .w = error bound (upper 16 bits, rounded up) | a | b << 5 | c << 10
+    float4 tf[CTM];       // vertex and its error bound
     float4 pf[CPM];       // FP32 planes (q, o)
     float4 cf[CCB];       // FP32 candidates (q, |q|^2 / 2)
     unsigned cid[CCB];    // sorted index | image code << 27
@@ -53,13 +54,13 @@ struct __align__(16) CellSmem {
     unsigned bm[CPM];     // removed directed edges
     unsigned pid[CPM];    // plane references: sorted index | image code << 27
     double off[9];        // image offsets s L - p: off[3 d + s + 1]
-    float tr2[CTM];       // upper bound of |v|^2
     float offf[9];
+    unsigned short vtri[CTM]; // the vertices' triangles a | b << 5 | c << 10
     unsigned short tri[CNS];  // new triangles
-    unsigned short rem[CNS];  // removed triangles
-    unsigned char hole[CNS];  // and their places
+    unsigned char hole[CNS];  // removed vertices
     unsigned char bcode[32];  // sx | sy << 2 | sz << 4 | self << 6 of the bins
     unsigned char perm[CCB];  // candidates in order
+    int pad[5];
 };
 // eight blocks of two warps (eight cells each) an SM; the cells of a warp start in different banks
 static_assert(sizeof(CellSmem) % 32 == 16 && 8 * (8 * sizeof(CellSmem) + 1024) <= 228 * 1024, "shared memory of a cell");
@@ -75,8 +76,8 @@ __device__ __forceinline__ float sqrt_fast(float x)
 // chunks of 32 of the (2r+1)^3 block: offsets + 8 as x | y << 4 | z << 8, and
 // where each chunk starts.
 struct Shells {
-    unsigned short bin[9 * 9 * 9];
-    unsigned short chunk[64];   // first entry of chunk c (all shells' chunks in a row)
+    unsigned short bin[13 * 13 * 13];
+    unsigned short chunk[160];  // first entry of chunk c (all shells' chunks in a row)
     unsigned char first[CELL_RINGS + 2];  // first chunk of shell r
 };
 constexpr Shells make_shells()
@@ -99,13 +100,6 @@ constexpr Shells make_shells()
     return t;
 }
 __device__ const Shells SHELLS = make_shells();
-
-__device__ __forceinline__ unsigned tri_of(float w) { return __float_as_uint(w) & 0x7fffu; }
-// error bound rounded up to 16 bits, with the triangle below
-__device__ __forceinline__ float pack_w(float err, unsigned tri)
-{
-    return __uint_as_float(((__float_as_uint(err) + 0xffffu) & 0xffff0000u) | tri);
-}
 
 // FP64 plane of a reference: q = r_j + s L - p and o = |q|^2 / 2.
 __device__ __forceinline__ void plane64(const double *off, unsigned ref, const double4_32a *__restrict__ sorted,
@@ -211,7 +205,7 @@ __device__ __noinline__ void fill_holes(CellSmem &S, int nnew, int nrem, int nt)
         if (!((holes >> e) & 1ull)) {
             const int h = __ffsll((long long)holes) - 1;
             S.tf[h] = S.tf[e];
-            S.tr2[h] = S.tr2[e];
+            S.vtri[h] = S.vtri[e];
             holes &= holes - 1ull;
         } else {
             holes &= ~(1ull << e);
@@ -367,13 +361,13 @@ warp_geometry(GeomSmem &S, int lane, int64_t w0, int w, int nt, const BoxDev *gp
                 const int p = __ffs((int)r) - 1, k = pb + __popc(lv & ((1u << p) - 1u));
                 if ((k & (TEAM - 1)) == tl) S.item[k] = (unsigned short)(tc << 5 | p);
             }
-#pragma unroll 2
+#pragma unroll 1
             for (int t = tl; t < nt; t += TEAM) S.vitem[vb + t] = (unsigned short)(tc << 6 | t);
         }
         if (lane < 16) S.hist[lane] = 0;
         {
             uint4 *const z = reinterpret_cast<uint4 *>(&S.nxt[0][0]);
-#pragma unroll 2
+#pragma unroll 1
             for (int i = lane; i < npl * CPM / 16; i += 32) z[i] = make_uint4(FULL, FULL, FULL, FULL);
         }
         __syncwarp();
@@ -523,27 +517,21 @@ warp_geometry(GeomSmem &S, int lane, int64_t w0, int w, int nt, const BoxDev *gp
         double a0, a1, a2, a3;
         {
             const unsigned lv = S.live[tc];
-            double b[2][4];
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                double s[2][4];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int p = tl + 8 * g + 16 * e;
-                    const bool has = mine && ((lv >> p) & 1u);
-                    const int k = has ? pb + __popc(lv & ((1u << p) - 1u)) : 0;
-                    s[e][0] = has ? S.vp[k] : 0.0;
-                    s[e][1] = has ? S.py[k] : 0.0;
-                    s[e][2] = has ? S.pz[k] : 0.0;
-                    s[e][3] = has ? S.po[k] : 0.0;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) b[g][q] = __dadd_rn(s[0][q], s[1][q]);
+            a0 = a1 = a2 = a3 = 0.0;
+#pragma unroll 1
+            for (int p = tl; p < 16; p += 8) {
+                const bool lo = mine && ((lv >> p) & 1u), hi = mine && ((lv >> (p + 16)) & 1u);
+                const int k = lo ? pb + __popc(lv & ((1u << p) - 1u)) : 0;
+                const int h = hi ? pb + __popc(lv & ((1u << (p + 16)) - 1u)) : 0;
+                const double b0 = __dadd_rn(lo ? S.vp[k] : 0.0, hi ? S.vp[h] : 0.0);
+                const double b1 = __dadd_rn(lo ? S.py[k] : 0.0, hi ? S.py[h] : 0.0);
+                const double b2 = __dadd_rn(lo ? S.pz[k] : 0.0, hi ? S.pz[h] : 0.0);
+                const double b3 = __dadd_rn(lo ? S.po[k] : 0.0, hi ? S.po[h] : 0.0);
+                a0 = __dadd_rn(a0, b0);  // (0 + b is b)
+                a1 = __dadd_rn(a1, b1);
+                a2 = __dadd_rn(a2, b2);
+                a3 = __dadd_rn(a3, b3);
             }
-            a0 = __dadd_rn(b[0][0], b[1][0]);
-            a1 = __dadd_rn(b[0][1], b[1][1]);
-            a2 = __dadd_rn(b[0][2], b[1][2]);
-            a3 = __dadd_rn(b[0][3], b[1][3]);
         }
         // each exchange halves the sums a lane keeps: lanes 0-1 of the eight end
         // with the volume, 2-3, 4-5 and 6-7 with the moment's components
@@ -572,6 +560,25 @@ warp_geometry(GeomSmem &S, int lane, int64_t w0, int w, int nt, const BoxDev *gp
         todo = todo && !mine;
         __syncwarp();
     }
+}
+
+// Largest |v|^2 bound of a cell's vertices, (|v| + err)^2 <= |v|^2 + err (2 |v|_1 + err).
+// Formed when candidates are gathered or screened, not at every cut.
+template <int G>
+__device__ __forceinline__ float r2_max(const CellSmem &S, int nt, int gl)
+{
+    float mr = 0.0f;
+#pragma unroll 1
+    for (int t = gl; t < nt; t += G) {
+        const float4 V = S.tf[t];
+        const float s2 = fmaf(V.x, V.x, fmaf(V.y, V.y, V.z * V.z)), l1 = fabsf(V.x) + fabsf(V.y) + fabsf(V.z);
+        // (a corner of the starting box has no error; the factors are k_clip's, so
+        // that the same candidates are gathered)
+        mr = fmaxf(mr, fmaf(V.w, fmaf(2.0f, l1, V.w), s2) * (V.w == 0.0f ? 1.000001f : 1.00001f));
+    }
+#pragma unroll
+    for (int o = G / 2; o >= 1; o >>= 1) mr = fmaxf(mr, __shfl_xor_sync(FULL, mr, o));
+    return mr;
 }
 
 template <int G>
@@ -623,8 +630,8 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
             unsigned a = sx, b = 2 + sy, c = 4 + sz;
             if ((sx ^ sy ^ sz) & 1) { const unsigned t = b; b = c; c = t; }
             const float x = 0.5f * (sx ? -L0 : L0), y = 0.5f * (sy ? -L1 : L1), z = 0.5f * (sz ? -L2 : L2);
-            S.tr2[gl] = fmaf(x, x, fmaf(y, y, z * z)) * 1.000001f;
-            S.tf[gl] = make_float4(x, y, z, pack_w(0.0f, a | (b << 5) | (c << 10)));
+            S.tf[gl] = make_float4(x, y, z, 0.0f);
+            S.vtri[gl] = (unsigned short)(a | (b << 5) | (c << 10));
         }
         lim4 = fmaf(L0, L0, fmaf(L1, L1, L2 * L2)) * 1.000001f;
         slack = 2e-6f * fmaxf(L0, fmaxf(L1, L2));
@@ -773,6 +780,10 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
         while (__any_sync(FULL, run && k < mc)) {
             const bool scr = run && k >= fit && k < mc;
             if (__any_sync(FULL, scr)) {
+                {
+                    const float r2 = r2_max<G>(S, nt, gl);
+                    if (np > 6) lim4 = 4.0f * r2;
+                }
                 const int cnt = scr ? mc - k : 0, maxc = __reduce_max_sync(FULL, cnt);
                 int dst = k;
 #pragma unroll 1
@@ -784,7 +795,7 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
                         if (2.0f * F.w <= lim4 * 1.000001f) {
                             const float qn = sqrt_fast(2.0f * F.w) * 1.00003f;
                             float far = -__int_as_float(0x7f800000);
-#pragma unroll 2
+#pragma unroll 1
                             for (int t = 0; t < nt; ++t) {
                                 const float4 V = S.tf[t];
                                 const float s = fmaf(F.x, V.x, fmaf(F.y, V.y, fmaf(F.z, V.z, -F.w)));
@@ -820,7 +831,7 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
                         const float cst = F.w > 1e-30f ? 16.0f * 5.9604645e-8f * 1.0001f * fmaf(qn, rmax, F.w)
                                                        : __int_as_float(0x7f800000);
                         unsigned bit = 1u;
-#pragma unroll 2
+#pragma unroll 1
                         for (int t = gl; t < nt; t += G, bit <<= 1) {
                             const float4 V = S.tf[t];
                             const float s = fmaf(F.x, V.x, fmaf(F.y, V.y, fmaf(F.z, V.z, -F.w)));
@@ -835,7 +846,7 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
                     while (um) {
                         const int c = __ffs((int)um) - 1;
                         um &= um - 1u;
-                        if (beyond_ref(S, tri_of(S.tf[c * G + gl].w), S.cid[kk], sorted, gp)) my |= 1u << c;
+                        if (beyond_ref(S, S.vtri[c * G + gl], S.cid[kk], sorted, gp)) my |= 1u << c;
                     }
                     __syncwarp();
                 }
@@ -862,11 +873,8 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
             while (my) {
                 const int t = (__ffs((int)my) - 1) * G + gl;
                 my &= my - 1u;
-                const unsigned v = tri_of(S.tf[t].w);
-                if (pos < CNS) {
-                    S.rem[pos] = (unsigned short)v;
-                    S.hole[pos] = (unsigned char)t;
-                }
+                const unsigned v = S.vtri[t];
+                if (pos < CNS) S.hole[pos] = (unsigned char)t;
                 ++pos;
                 const unsigned x = v & 31u, y = (v >> 5) & 31u, z = v >> 10;
                 atomicOr(&S.bm[x], 1u << y);
@@ -880,7 +888,7 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
                 unsigned live = 0;
 #pragma unroll 1
                 for (int t = gl; t < nt; t += G) {
-                    const unsigned v = tri_of(S.tf[t].w);
+                    const unsigned v = S.vtri[t];
                     live |= (1u << (v & 31u)) | (1u << ((v >> 5) & 31u)) | (1u << (v >> 10));
                 }
 #pragma unroll
@@ -905,7 +913,7 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
                 unsigned x = 0, y = 0, z = 0;
                 bool f0 = false, f1 = false, f2 = false;
                 if (go && i < nrem) {
-                    const unsigned v = S.rem[i];
+                    const unsigned v = S.vtri[S.hole[i]];
                     x = v & 31u, y = (v >> 5) & 31u, z = v >> 10;
                     f0 = !((S.bm[y] >> x) & 1u);
                     f1 = !((S.bm[z] >> y) & 1u);
@@ -951,11 +959,9 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
                         x = (float)X.x; y = (float)X.y; z = (float)X.z;
                         er = 1.2e-7f * (fabsf(x) + fabsf(y) + fabsf(z)) + 1e-38f;
                     }
-                    const float s2 = fmaf(x, x, fmaf(y, y, z * z));
-                    const float l1 = fabsf(x) + fabsf(y) + fabsf(z);
                     const int t = i < nrem ? (int)S.hole[i] : nt + i - nrem;
-                    S.tf[t] = make_float4(x, y, z, pack_w(er, v));
-                    S.tr2[t] = fmaf(er, fmaf(2.0f, l1, er), s2) * 1.00001f;
+                    S.tf[t] = make_float4(x, y, z, er);
+                    S.vtri[t] = (unsigned short)v;
                 }
             }
             __syncwarp();
@@ -968,12 +974,10 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
                 np = max(np, kp + 1);
                 ++k;
             }
-            float mr = 0.0f;
-#pragma unroll 2
-            for (int t = gl; t < nt; t += G) mr = fmaxf(mr, S.tr2[t]);
-#pragma unroll
-            for (int o = G / 2; o >= 1; o >>= 1) mr = fmaxf(mr, __shfl_xor_sync(FULL, mr, o));
-            if (go) lim4 = 4.0f * mr;
+        }
+        {
+            const float r2 = r2_max<G>(S, nt, gl);
+            if (np > 6) lim4 = 4.0f * r2;
         }
         // bins are passed over, and rmax bounds |v|, by an earlier limit: it may
         // not grow past their margins (it shrinks but for the error bounds)
@@ -1017,7 +1021,7 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
         for (int r = 0; r < NP; ++r) ref[r] = S.pid[r * G + gl];
 #pragma unroll
         for (int r = 0; r < NV; ++r) {
-            const unsigned v = tri_of(S.tf[r * G + gl].w);
+            const unsigned v = S.vtri[r * G + gl];
             tri[r] = v;
             if (r * G + gl < nt) lv |= (1u << (v & 31u)) | (1u << ((v >> 5) & 31u)) | (1u << (v >> 10));
         }

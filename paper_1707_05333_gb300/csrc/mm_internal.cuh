@@ -27,10 +27,10 @@ constexpr int PMAX_BIG = 128, TMAX_BIG = 256, NSTAGE_BIG = 64, MAXF_BIG = 128, M
 constexpr int CLIP_MAX_WARPS = 8;  // warps (cells) per block of the clipper, tunable at run time
 // Cells from which the grouped clipper (mm_cells.cu) runs.  Below, the chip is
 // not full and a warp per cell finishes sooner.  Tessellation, warp per cell
-// against grouped: 1000 random generators 0.29 / 0.40 ms, 4100 0.43 / 0.60,
-// 8000 0.65 / 0.65, 16000 0.99 / 0.87, 200003 9.5 / 5.4; jittered lattices 20^3
-// 0.38 / 0.28, 64^3 6.4 / 3.6.
-constexpr int64_t CELLS_MIN = 8000;
+// against grouped: 2000 random generators 0.35 / 0.41 ms, 4100 0.44 / 0.45,
+// 8000 0.65 / 0.48, 200003 9.6 / 4.9; jittered lattices 12^3 0.20 / 0.23,
+// 16^3 0.27 / 0.24, 20^3 0.38 / 0.27, 64^3 6.3 / 3.2.
+constexpr int64_t CELLS_MIN = 4096;
 // Overflow rows reserved when the count of retried cells is not known in
 // advance (graph mode); mm_tessellate sizes them to the count it reads.
 constexpr int RETRY_ROWS_FIXED = 256;

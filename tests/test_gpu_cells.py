@@ -1,4 +1,4 @@
-"""The grouped clipper (several cells to a warp, 8000 cells and more) against
+"""The grouped clipper (several cells to a warp, 4096 cells and more) against
 the warp-per-cell filtered clipper, which runs when the work counters are on:
 the same mesh, bit for bit.  (The direct FP64 clipper forms its search limit in
 FP64 and may meet candidates in other batches, which orders a cell's faces
@@ -37,6 +37,9 @@ def sheet(n):
 
 CASES = {
     # the rule's edge, and counts that fill the warps of four and of eight cells unevenly
+    "random_4095": lambda: (WL.random_points(4095, seed=33), np.ones(3)),
+    "random_4096": lambda: (WL.random_points(4096, seed=34), np.ones(3)),
+    "random_4099": lambda: (WL.random_points(4099, seed=35), np.ones(3)),
     "random_7999": lambda: (WL.random_points(7999, seed=21), np.ones(3)),
     "random_8000": lambda: (WL.random_points(8000, seed=22), np.ones(3)),
     "random_8003": lambda: (WL.random_points(8003, seed=23), np.ones(3)),
