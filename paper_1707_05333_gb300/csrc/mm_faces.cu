@@ -298,8 +298,9 @@ void launch_face_confirm(int64_t n, Slots sl, OvfFaces ov, const BoxDev *boxes, 
                          unsigned long long *emit_mask, unsigned long long *conf_mask, signed char *partner,
                          int *emit_cnt, int *conf_cnt, cudaStream_t s)
 {
-    const int64_t nb = (n * CONFIRM_LANES + 127) / 128;
-    k_face_confirm<<<(unsigned)nb, 128, 0, s>>>(n, sl, ov, boxes, cbox, st, emit_mask, conf_mask, partner, emit_cnt,
+    const int bs = spread_block(n * CONFIRM_LANES, 128);
+    const int64_t nb = (n * CONFIRM_LANES + bs - 1) / bs;
+    k_face_confirm<<<(unsigned)nb, bs, 0, s>>>(n, sl, ov, boxes, cbox, st, emit_mask, conf_mask, partner, emit_cnt,
                                                 conf_cnt);
 }
 
@@ -310,8 +311,8 @@ void launch_face_write(int64_t n, const double *pos, const BoxDev *boxes, const 
                        int64_t fcap, int *inc_face, int64_t icap, const double *vol, double *cen, DevStatus *st,
                        cudaStream_t s)
 {
-    const int nb = (int)((n + 31) / 32);  // 32 cells per block of 128 threads
-    k_face_write<<<nb, 128, 0, s>>>(n, pos, boxes, cbox, sl, ov, emit_mask, conf_mask, partner, face_off, inc_off,
+    const int bs = spread_block(4 * n, 128), nb = (int)((4 * n + bs - 1) / bs);
+    k_face_write<<<nb, bs, 0, s>>>(n, pos, boxes, cbox, sl, ov, emit_mask, conf_mask, partner, face_off, inc_off,
                                     face_i, face_j, face_shift, face_area, face_normal, face_cen, fcap, inc_face,
                                     icap, vol, cen, st);
 }

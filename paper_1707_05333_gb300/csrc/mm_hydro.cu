@@ -89,6 +89,24 @@ __device__ __forceinline__ double deldot(double g0, double g1, double g2, double
 }
 __device__ __forceinline__ long long kmin(long long a, long long b) { return a < b ? a : b; }
 
+// The face of an incidence, its side and the cell across.  The loops over a
+// cell's faces fetch the next one's before they work on this one: the loads
+// hang on one another (incidence, face, neighbour's state) and a thread would
+// wait for each in turn.
+struct Across {
+    int f, o;
+    bool fwd;
+};
+__device__ __forceinline__ Across across(const MeshDev &m, int e)
+{
+    Across a;
+    const int f = m.inc_face[e];
+    a.fwd = f >= 0;
+    a.f = a.fwd ? f : ~f;
+    a.o = a.fwd ? m.face_j[a.f] : m.face_i[a.f];
+    return a;
+}
+
 // ---------------------------------------------------------------------------
 // Gradient + limiter (+ half-step predictor when PREDICT)
 // ---------------------------------------------------------------------------
@@ -121,12 +139,11 @@ __global__ void __launch_bounds__(128, MM_GRAD_MINBLOCKS) k_gradient(MeshDev m, 
     for (int k = 0; k < NG; ++k) { kx[k] = okey(Wi[k]); kn[k] = kx[k]; }
 #pragma unroll
     for (int k = 0; k < 3 * NG; ++k) b[k] = 0.0;
+    Across next = e0 < e1 ? across(m, e0) : Across{0, 0, true};
     for (int e = e0; e < e1; ++e) {
-        int f = m.inc_face[e];
-        const bool fwd = f >= 0;
-        if (!fwd) f = ~f;
-        const int o = fwd ? m.face_j[f] : m.face_i[f];
-        const long long sm = fwd ? 0LL : (long long)0x8000000000000000ULL;
+        const int f = next.f, o = next.o;
+        const long long sm = next.fwd ? 0LL : (long long)0x8000000000000000ULL;
+        if (e + 1 < e1) next = across(m, e + 1);
         const double ax = geo[f], ay = geo[fs + f], az = geo[2 * fs + f];
         if (!MINV_IN) {
             const double dx = geo[3 * fs + f], dy = geo[4 * fs + f], dz = geo[5 * fs + f];
@@ -200,8 +217,10 @@ __global__ void __launch_bounds__(128, MM_GRAD_MINBLOCKS) k_gradient(MeshDev m, 
                 m2[k] = -__int_as_float(0x7f800000); n2[k] = __int_as_float(0x7f800000);
             }
             float dl1 = 0.0f;
+            int fn = e0 < e1 ? m.inc_face[e0] : 0;
             for (int e = e0; e < e1; ++e) {
-                int f = m.inc_face[e];
+                int f = fn;
+                if (e + 1 < e1) fn = m.inc_face[e + 1];
                 const unsigned sm = f >= 0 ? 0u : 0x80000000u;
                 if (f < 0) f = ~f;
                 const float dx = __uint_as_float(__float_as_uint(g32[f]) ^ sm);
@@ -393,10 +412,10 @@ template <int NG>
 static void launch_gradient_t(const MeshDev &m, const HydroCfg &c, const double *W, const double *geo, double *minv,
                               bool minv_in, double *grad, double *W_half, const double *dt, cudaStream_t s)
 {
-    const int nb = (int)((m.n + 127) / 128);
-    if (W_half) k_gradient<true, false, NG><<<nb, 128, 0, s>>>(m, c, W, geo, minv, grad, W_half, dt);
-    else if (minv_in) k_gradient<false, true, NG><<<nb, 128, 0, s>>>(m, c, W, geo, minv, grad, W_half, dt);
-    else k_gradient<false, false, NG><<<nb, 128, 0, s>>>(m, c, W, geo, minv, grad, W_half, dt);
+    const int bs = spread_block(m.n, 128), nb = (int)((m.n + bs - 1) / bs);
+    if (W_half) k_gradient<true, false, NG><<<nb, bs, 0, s>>>(m, c, W, geo, minv, grad, W_half, dt);
+    else if (minv_in) k_gradient<false, true, NG><<<nb, bs, 0, s>>>(m, c, W, geo, minv, grad, W_half, dt);
+    else k_gradient<false, false, NG><<<nb, bs, 0, s>>>(m, c, W, geo, minv, grad, W_half, dt);
 }
 
 void launch_gradient(const MeshDev &m, const HydroCfg &c, const double *W, const double *geo, double *minv,
@@ -539,8 +558,11 @@ __global__ void __launch_bounds__(256) k_update(MeshDev m, HydroCfg c, const dou
 #pragma unroll
     for (int k = 0; k < NG; ++k) acc[k] = 0.0;
     double mc = 0.0, dv = 0.0;
-    for (int e = m.inc_off[i]; e < m.inc_off[i + 1]; ++e) {
-        int f = m.inc_face[e];
+    const int e1 = m.inc_off[i + 1];
+    int e = m.inc_off[i], fn = e < e1 ? m.inc_face[e] : 0;
+    for (; e < e1; ++e) {
+        int f = fn;
+        if (e + 1 < e1) fn = m.inc_face[e + 1];
         double sg = 1.0;
         if (f < 0) { f = ~f; sg = -1.0; }
 #pragma unroll
@@ -594,9 +616,9 @@ __global__ void __launch_bounds__(256) k_update(MeshDev m, HydroCfg c, const dou
 void launch_update(const MeshDev &m, const HydroCfg &c, const double *flux, const double *dt, double *U,
                    cudaStream_t s)
 {
-    int nb = (int)((m.n + 255) / 256);
-    if (c.entropy) k_update<6><<<nb, 256, 0, s>>>(m, c, flux, dt, U);
-    else k_update<5><<<nb, 256, 0, s>>>(m, c, flux, dt, U);
+    const int bs = spread_block(m.n, 256), nb = (int)((m.n + bs - 1) / bs);
+    if (c.entropy) k_update<6><<<nb, bs, 0, s>>>(m, c, flux, dt, U);
+    else k_update<5><<<nb, bs, 0, s>>>(m, c, flux, dt, U);
 }
 
 // ---------------------------------------------------------------------------
@@ -746,8 +768,8 @@ void launch_dt_init(double *dt, int nbox, cudaStream_t s) { k_dt_init<<<(nbox + 
 void launch_mesh_velocity(const MeshDev &m, const HydroCfg &c, const double *pos, const double *U, double *w,
                           double *dt_min, cudaStream_t s)
 {
-    int nb = (int)((m.n + 255) / 256);
-    k_mesh_velocity<<<nb, 256, 0, s>>>(m, c, pos, U, w, reinterpret_cast<unsigned long long *>(dt_min));
+    const int bs = spread_block(m.n, 256), nb = (int)((m.n + bs - 1) / bs);
+    k_mesh_velocity<<<nb, bs, 0, s>>>(m, c, pos, U, w, reinterpret_cast<unsigned long long *>(dt_min));
 }
 
 // ---------------------------------------------------------------------------

@@ -354,22 +354,23 @@ __global__ void __launch_bounds__(256) k_update32(MeshDev m, HydroCfg c, Mixed x
 void launch_mixed_step(const MeshDev &m, const HydroCfg &c, const double *pos, const double *w, const double *dt,
                        Mixed x, double *U, cudaStream_t s, void (*mark)(void *, int, bool), void *mark_arg)
 {
-    const int nbc = (int)((m.n + 127) / 128), nbc2 = (int)((m.n + 255) / 256);
+    const int bsg = spread_block(m.n, 128), nbc = (int)((m.n + bsg - 1) / bsg), nbc2 = (int)((m.n + 255) / 256);
+    const int bsu = spread_block(m.n, 256), nbu = (int)((m.n + bsu - 1) / bsu);
     const int64_t nfl = face_launch_count(m);
     const int nbf = (int)((nfl + 255) / 256), nbf2 = (int)((nfl + 127) / 128);
     mark(mark_arg, MM_STAGE_GRADIENT_HALF, true);
     if (nfl > 0) k_faces32<<<nbf, 256, 0, s>>>(m, pos, x);
     k_pack32<<<nbc2, 256, 0, s>>>(m, U, pos, w, x);
-    k_gradient32<true><<<nbc, 128, 0, s>>>(m, c, x, x.cw, x.ch, dt);
+    k_gradient32<true><<<nbc, bsg, 0, s>>>(m, c, x, x.cw, x.ch, dt);
     mark(mark_arg, MM_STAGE_GRADIENT_HALF, false);
     mark(mark_arg, MM_STAGE_GRADIENT, true);
-    k_gradient32<false><<<nbc, 128, 0, s>>>(m, c, x, x.ch, nullptr, dt);
+    k_gradient32<false><<<nbc, bsg, 0, s>>>(m, c, x, x.ch, nullptr, dt);
     mark(mark_arg, MM_STAGE_GRADIENT, false);
     mark(mark_arg, MM_STAGE_FACE_FLUX, true);
     if (nfl > 0) k_face_flux32<<<nbf2, 128, 0, s>>>(m, c, x);
     mark(mark_arg, MM_STAGE_FACE_FLUX, false);
     mark(mark_arg, MM_STAGE_UPDATE, true);
-    k_update32<<<nbc2, 256, 0, s>>>(m, c, x, dt, U);
+    k_update32<<<nbu, bsu, 0, s>>>(m, c, x, dt, U);
     mark(mark_arg, MM_STAGE_UPDATE, false);
 }
 

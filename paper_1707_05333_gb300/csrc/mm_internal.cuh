@@ -24,6 +24,7 @@ constexpr int NSTAGE = 32;  // vertices created by one cut
 constexpr int MAXF = 48;    // faces written per cell
 constexpr int MAXRING = 48; // search rings before giving up
 constexpr int PMAX_BIG = 128, TMAX_BIG = 256, NSTAGE_BIG = 64, MAXF_BIG = 128, MAXRING_BIG = 128;
+constexpr int NUM_SMS = 152;       // GB300
 constexpr int CLIP_MAX_WARPS = 8;  // warps (cells) per block of the clipper, tunable at run time
 // Cells from which the grouped clipper (mm_cells.cu) runs.  Below, the chip is
 // not full and a warp per cell finishes sooner.  Tessellation, warp per cell
@@ -103,6 +104,17 @@ struct OvfFaces {
     signed char *partner;             // [orows*MAXF_BIG]
     const int *nretry;                // cells re-clipped (0: no overflow row is in use)
 };
+
+// Threads per block of a kernel of `threads` independent threads: its usual
+// block, or less (down to a warp) where that leaves SMs without one: a 16^3
+// box has 32 blocks of 128 threads.  With the look-ahead of the face loops
+// (across in mm_hydro.cu) steps of 4096 to 53000 cells gain 0.6 to 0.8 %.
+inline int spread_block(int64_t threads, int usual)
+{
+    int b = usual;
+    while (b > 32 && threads < (int64_t)b * NUM_SMS * 2) b >>= 1;
+    return b;
+}
 
 // kernels' host launchers (stream-ordered, no syncs)
 void launch_fill_cbox(const long long *box_off, int nbox, int64_t n, int *cbox, cudaStream_t s);
