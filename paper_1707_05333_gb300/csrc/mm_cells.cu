@@ -10,15 +10,19 @@
 //
 // What bounds it and what it measured (GB300, jittered 64^3 lattice and
 // 200003 random generators, ncu durations; k_clip took 5.89 and 8.89 ms):
-// 2.73 and 4.26 ms, of dependent latencies with 15 warps an SM (3.4 KB of
+// 2.6 and 4.2 ms, of dependent latencies with 15 warps an SM (3.4 KB of
 // shared memory a cell, 128 registers): 1.6 instructions a cycle, 5220 a cell
 // against k_clip's 14200, and the FP64 pipe 52 % busy with 107 instructions a
 // cell against 236.  (18 warps an SM at 96 registers gained nothing: the
 // misses of the instruction cache doubled.)
 //  * Loops are kept rolled: unrolled, the body outgrew the instruction cache
 //    and half of the cycles went to fetching it (5.3 and 13.0 ms).
-//  * Screening candidates a lane each after the first 16 instead of trying all
-//    one by one: random generators 4.33 -> 3.58 ms (clipping alone).
+//  * Screening candidates a lane each after the first SCREEN instead of trying
+//    all one by one: random generators 4.33 -> 3.58 ms (clipping alone).
+//  * The library's divisions, for the ends of the range only, stand out of line:
+//    tessellation of a 128^3 lattice 24.5 -> 24.0 ms.  Unrolling the vertex loop
+//    twice, or the plane-test loop four times, costs 11 and 4 % for the
+//    instruction cache.
 //  * The geometry as a kernel of its own (1.45 and 1.10 ms, FP64 pipe 84 %
 //    busy, after 1.70 and 3.58 ms of clipping) left the FP64 pipe idle in one
 //    kernel and the issue slots in the other: 3.15 and 4.68 ms in all, here
@@ -39,7 +43,7 @@ constexpr int CTM = 56;    // vertices
 constexpr int CNS = 32;    // new (and removed) vertices of one cut
 constexpr int CCB = 64;    // candidate buffer, flushed as in k_clip
 constexpr int CELL_RINGS = 6;
-constexpr int SCREEN = 16;
+constexpr int SCREEN = 8;     // candidates of a new cell tried unscreened (16: 2.7 % slower on lattices, 4: 4 %)
 constexpr int LANES = 8;   // lanes a cell (16 lanes: jittered 64^3 2.35 ms for 1.70, random generators the same)
 constexpr unsigned BOX_PLANE = 31u << 27;  // plane reference of box face k: BOX_PLANE | k
 constexpr unsigned IDX_MASK = 0x7ffffffu;  // sorted index of a plane reference (MM_MAX_CELLS < 2^27)
@@ -670,7 +674,7 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
             const bool setup = act && !any;
             if (__any_sync(FULL, setup)) {
                 // the chunk's bins that hold generators within reach, in order
-                const float reach = 1.02f * fmaf(slack, sqrtf(limk), limk);
+                const float reach = 1.02f * fmaf(slack, sqrt_fast(limk), limk);
                 const int b0 = SHELLS.chunk[chunk], nb = setup ? SHELLS.chunk[chunk + 1] - b0 : 0;
                 const int maxnb = __reduce_max_sync(FULL, nb);
                 int found = 0, most = 0;

@@ -16,9 +16,14 @@ __device__ __forceinline__ bool seed_range(double x)
     return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 23u < 2000u;
 }
 
+// The library's operations, out of line: they are for the ends of the range only
+static __device__ __noinline__ double rcp_any(double x) { return 1.0 / x; }
+static __device__ __noinline__ double quot_any(double a, double b) { return a / b; }
+static __device__ __noinline__ double rsqrt_any(double x) { return rsqrt(x); }
+
 __device__ __forceinline__ double rcp64(double x)
 {
-    if (!seed_range(x)) return 1.0 / x;
+    if (!seed_range(x)) return rcp_any(x);
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = __fma_rn(-x, y, 1.0);
@@ -31,13 +36,13 @@ __device__ __forceinline__ double div64(double a, double b)
     const double y = rcp64(b), q = __dmul_rn(a, y);
     const double r = __fma_rn(__fma_rn(-b, q, a), y, q);
     // a quotient near the range's ends (zero is exact): the library's
-    return seed_range(q) || (__double_as_longlong(q) << 1) == 0 ? r : a / b;
+    return seed_range(q) || (__double_as_longlong(q) << 1) == 0 ? r : quot_any(a, b);
 }
 
 // 1 / sqrt(x), x > 0: with e = 1 - x y^2, y (1 + e/2 + 3 e^2 / 8)
 __device__ __forceinline__ double rsqrt64(double x)
 {
-    if (!seed_range(x)) return rsqrt(x);
+    if (!seed_range(x)) return rsqrt_any(x);
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
