@@ -7,6 +7,7 @@
 // code is above the zero-shift code.  Offsets come from exclusive scans of
 // per-cell counts, so face ids and every cell's incident list are
 // deterministic: no atomics on the data path.
+#include "mm_fp64.cuh"
 #include "mm_internal.cuh"
 
 namespace mm {
@@ -213,15 +214,16 @@ __device__ __forceinline__ void face_write_slots(int64_t n, int64_t i, int lane,
         if ((((k < 64 ? em0 : em1) >> (k & 63)) & 1ull)) {
             const int f = fbase + (OVF ? popc_below(em0, em1, k) : __popcll(em0 & ((1ull << k) - 1ull)));
             if (f < fcap) {
-                // image offsets -L, 0, +L by selection (no FP64 arithmetic)
-                const int cx = code % 3, cy = (code / 3) % 3, cz = code / 9;
-                const double ox = cx == 1 ? 0.0 : (cx == 2 ? L[0] : -L[0]);
-                const double oy = cy == 1 ? 0.0 : (cy == 2 ? L[1] : -L[1]);
-                const double oz = cz == 1 ? 0.0 : (cz == 2 ? L[2] : -L[2]);
-                const double qx = pos[j] + ox - pix;
-                const double qy = pos[n + j] + oy - piy;
-                const double qz = pos[2 * n + j] + oz - piz;
-                const double inv = rsqrt(qx * qx + qy * qy + qz * qz);
+                // image offsets -L, +L by selection (no FP64 arithmetic), none inside the box
+                double pjx = pos[j], pjy = pos[n + j], pjz = pos[2 * n + j];
+                if (code != 13) {
+                    const int cx = code % 3, cy = (code / 3) % 3, cz = code / 9;
+                    pjx += cx == 1 ? 0.0 : (cx == 2 ? L[0] : -L[0]);
+                    pjy += cy == 1 ? 0.0 : (cy == 2 ? L[1] : -L[1]);
+                    pjz += cz == 1 ? 0.0 : (cz == 2 ? L[2] : -L[2]);
+                }
+                const double qx = pjx - pix, qy = pjy - piy, qz = pjz - piz;
+                const double inv = rsqrt64(qx * qx + qy * qy + qz * qz);
                 face_i[f] = (int)i;
                 face_j[f] = j;
                 face_shift[f] = code;
@@ -273,7 +275,7 @@ __global__ void k_face_write(int64_t n, const double *__restrict__ pos, const Bo
     if (lane == 0) {
         // the cell centroid from the clipper's volume and first moment about
         // the generator
-        const double ivl = 1.0 / vol[i];
+        const double ivl = rcp64(vol[i]);
         cen[i] = pix + cen[i] * ivl;
         cen[n + i] = piy + cen[n + i] * ivl;
         cen[2 * n + i] = piz + cen[2 * n + i] * ivl;

@@ -20,6 +20,7 @@ __device__ __forceinline__ bool seed_range(double x)
 static __device__ __noinline__ double rcp_any(double x) { return 1.0 / x; }
 static __device__ __noinline__ double quot_any(double a, double b) { return a / b; }
 static __device__ __noinline__ double rsqrt_any(double x) { return rsqrt(x); }
+static __device__ __noinline__ double sqrt_any(double x) { return sqrt(x); }
 
 __device__ __forceinline__ double rcp64(double x)
 {
@@ -45,8 +46,21 @@ __device__ __forceinline__ double rsqrt64(double x)
     if (!seed_range(x)) return rsqrt_any(x);
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    const double t = __dmul_rn(x, y);  // and its rounding, or e would carry it
+    const double e = __fma_rn(-__fma_rn(x, y, -t), y, __fma_rn(-t, y, 1.0));
     return __fma_rn(__dmul_rn(y, e), __fma_rn(e, 0.375, 0.5), y);
+}
+
+// sqrt(x): the same iteration on t = x y, then one residual step,
+// s + (x - s^2) y / 2 (y / 2 by its exponent: y is a normal number)
+__device__ __forceinline__ double sqrt64(double x)
+{
+    if (!seed_range(x) || __double_as_longlong(x) < 0) return sqrt_any(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double t = __dmul_rn(x, y), e = __fma_rn(-t, y, 1.0);
+    const double s = __fma_rn(__dmul_rn(t, e), __fma_rn(e, 0.375, 0.5), t);
+    return __fma_rn(__fma_rn(-s, s, x), __longlong_as_double(__double_as_longlong(y) - (1LL << 52)), s);
 }
 
 }  // namespace mm

@@ -53,14 +53,18 @@ __global__ void __launch_bounds__(256) k_face_geom(MeshDev m, double *__restrict
     const int64_t n = m.n, fs = m.fs;
     const int i = m.face_i[f], j = m.face_j[f];
     const int code = m.face_shift[f];
-    const double *L = m.boxL + 3 * m.cbox[i];
     const double A = m.area[f];
     geo[f] = A * m.normal[f];
     geo[fs + f] = A * m.normal[fs + f];
     geo[2 * fs + f] = A * m.normal[2 * fs + f];
-    const double dx = m.cen[j] + image_axis(code % 3, L[0]) - m.cen[i];
-    const double dy = m.cen[n + j] + image_axis((code / 3) % 3, L[1]) - m.cen[n + i];
-    const double dz = m.cen[2 * n + j] + image_axis(code / 9, L[2]) - m.cen[2 * n + i];
+    double cx = m.cen[j], cy = m.cen[n + j], cz = m.cen[2 * n + j];
+    if (code != 13) {  // a face inside the box adds no offset
+        const double *L = m.boxL + 3 * m.cbox[i];
+        cx += image_axis(code % 3, L[0]);
+        cy += image_axis((code / 3) % 3, L[1]);
+        cz += image_axis(code / 9, L[2]);
+    }
+    const double dx = cx - m.cen[i], dy = cy - m.cen[n + i], dz = cz - m.cen[2 * n + i];
     geo[3 * fs + f] = dx;
     geo[4 * fs + f] = dy;
     geo[5 * fs + f] = dz;

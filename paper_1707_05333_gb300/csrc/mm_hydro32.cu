@@ -32,12 +32,17 @@ __global__ void __launch_bounds__(256) k_faces32(MeshDev m, const double *__rest
     if (f >= face_count(m)) return;
     const int64_t n = m.n, fs = m.fs;
     const int i = m.face_i[f], j = m.face_j[f];
-    double sx, sy, sz;
-    decode_shift32(m.face_shift[f], sx, sy, sz);
-    const double *L = m.boxL + 3 * m.cbox[i];
-    const double qx = pos[j] + sx * L[0] - pos[i];
-    const double qy = pos[n + j] + sy * L[1] - pos[n + i];
-    const double qz = pos[2 * n + j] + sz * L[2] - pos[2 * n + i];
+    double pjx = pos[j], pjy = pos[n + j], pjz = pos[2 * n + j];
+    const int code = m.face_shift[f];
+    if (code != 13) {  // a face inside the box adds no offset
+        double sx, sy, sz;
+        decode_shift32(code, sx, sy, sz);
+        const double *L = m.boxL + 3 * m.cbox[i];
+        pjx += sx * L[0];
+        pjy += sy * L[1];
+        pjz += sz * L[2];
+    }
+    const double qx = pjx - pos[i], qy = pjy - pos[n + i], qz = pjz - pos[2 * n + i];
     const double fx = m.fcen[f] - pos[i], fy = m.fcen[fs + f] - pos[n + i], fz = m.fcen[2 * fs + f] - pos[2 * n + i];
     x.fij[f] = make_int2(i, j);
     x.fa[f] = make_float4((float)m.area[f], (float)m.normal[f], (float)m.normal[fs + f], (float)m.normal[2 * fs + f]);

@@ -46,7 +46,7 @@ __device__ __forceinline__ bool not_below_t(double a, double b)
     return okey(a) >= okey(b) && okey(a) <= inf;
 }
 __device__ __forceinline__ bool not_below_t(float a, float b) { return a >= b; }
-__device__ __forceinline__ double sqrt_t(double x) { return sqrt(x); }
+__device__ __forceinline__ double sqrt_t(double x) { return sqrt64(x); }
 __device__ __forceinline__ float sqrt_t(float x) { return sqrtf(x); }
 __device__ __forceinline__ double min_t(double a, double b) { return okey(a) < okey(b) ? a : b; }
 __device__ __forceinline__ float min_t(float a, float b) { return fminf(a, b); }
