@@ -174,7 +174,7 @@ def clip_roofline(direct, filtered, ms, n, clip_filter):
     plus its FP64 fallbacks, final solves and fans) is kept as an extra key."""
     f_method = clip_method_flops(direct)
     ach = f_method / (ms / 1e3) / 1e12
-    out = {"kernel": "k_clip", "bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS,
+    out = {"kernel": "k_cells" if clip_filter else "k_clip", "bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS,
            "unit": "TFLOP/s (FP64)", "frac": ach / FP64_PEAK_TFLOPS, "traffic": None,
            "peak_source": "derived: 152 SMs x 2 FP64 FMA lanes/clk x 2 flops x 2.07 GHz",
            "fp64_flops_per_launch": f_method, "fp64_flops_per_cell": f_method / n, "launch_ms": ms}
@@ -190,12 +190,13 @@ def clip_roofline(direct, filtered, ms, n, clip_filter):
     return out
 
 
-# DRAM traffic of the clipping kernels per cell, from an ncu capture of one
-# tessellation's launches.  Valid only for the clipper sources it was taken on:
-# the digest of the clipping kernels' sources must match, else the figure is
-# withheld.  (None: no capture of the current kernels.)
+# DRAM traffic of the clipper per cell, from an ncu capture of one k_cells launch
+# on the 128^3 shear layer (dram__bytes_read.sum + dram__bytes_write.sum = 452,787,968
+# + 1,435,980,800 bytes over 2,097,152 cells); it scales with the cells of the launch.
+# Valid only for the clipper sources it was taken on: the digest of the clipping
+# kernels' sources must match, else the figure is withheld.
 CLIP_TRAFFIC = {"sources": ("csrc/mm_cells.cu", "csrc/mm_clip.cu", "csrc/mm_clip.cuh", "csrc/mm_internal.cuh"),
-                "sha256_16": "", "bytes_per_cell": None, "cells_captured": 2097152}
+                "sha256_16": "317f07aec105e5f7", "bytes_per_cell": 1888768768 / 2097152, "cells_captured": 2097152}
 
 
 def clip_sources_digest():

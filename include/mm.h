@@ -73,7 +73,8 @@ typedef struct {
                       /*    FP64 update); the mesh is FP64-exact either way (clip_filter)   */
     int collect_stats;/* 1: the clipper records the counters read by mm_tess_stats          */
     int riemann;      /* 0 HLLC (the paper's default), 1 HLL (Sec. 4)                        */
-    int clip_warps;   /* cells (warps) per block of the clipping kernel, 1..8 (tunable; 2)   */
+    int clip_warps;   /* cells (warps) per block of the warp-per-cell clipper, 1..8 (tunable; */
+                      /*    2); from 4096 generators on it takes only the unusual cells      */
     int cand_cap;     /* candidates per sorted batch of the clipper, 32..64 (tunable)        */
     int clip_filter;  /* 1: clip with FP32 vertices, an error-bounded FP32 plane test and    */
                       /*    an exact FP64 test near ties, then FP64 vertices (same mesh, bit */
@@ -89,7 +90,7 @@ typedef struct {
     int integrator;   /* 0: half-step predictor with start-of-step geometry (Sec. 4.1);      */
                       /*    1: Heun, fluxes averaged over start and end meshes (Sec. 6; FP64 */
                       /*    hydro, no entropy column; one more tessellation per step)        */
-    int clip_sort;    /* how the clipper orders more than 32 buffered candidates: 0 in      */
+    int clip_sort;    /* how that clipper orders more than 32 buffered candidates: 0 in     */
                       /*    shared memory, 1 in registers (same order and mesh; tunable)      */
 } mm_config;
 
