@@ -39,11 +39,12 @@ __device__ __forceinline__ double inv_t(double x) { return rcp64(x); }
 __device__ __forceinline__ float inv_t(float x) { return 1.0f / x; }
 __device__ __forceinline__ double quot_t(double a, double b) { return div64(a, b); }
 __device__ __forceinline__ float quot_t(float a, float b) { return a / b; }
-// a >= b: FP64 by integers (false where either is NaN, as the operator)
+// a >= b: FP64 by integers (false where either is NaN, as the operator: a NaN's
+// key lies past the infinities' on its sign's side)
 __device__ __forceinline__ bool not_below_t(double a, double b)
 {
     const long long inf = 0x7ff0000000000000LL;
-    return okey(a) >= okey(b) && okey(a) <= inf;
+    return okey(a) >= okey(b) && okey(a) <= inf && okey(b) >= ~inf;
 }
 __device__ __forceinline__ bool not_below_t(float a, float b) { return a >= b; }
 __device__ __forceinline__ double sqrt_t(double x) { return sqrt64(x); }
