@@ -1,12 +1,14 @@
-// mm_fp64.cuh -- FP64 reciprocal, quotient and reciprocal square root by one
-// third-order iteration.
+// mm_fp64.cuh -- FP64 reciprocal, quotient, square root and its reciprocal by
+// one step of Chebyshev's third-order iteration.
 //
 // GB300 issues an FP64 instruction in 16 cycles of the SM's pipe, so their
 // number is what the kernels with FP64 arithmetic cost.  The hardware's seed
-// (rcp/rsqrt.approx.ftz.f64, about 20 good bits) with residual e = 1 - x y
-// gives 1/x = y / (1 - e) = y (1 + e + e^2) + O(e^3): 2^-60 relative, then one
-// rounding, in three instructions.  Outside 2^+-1000 the seed would flush and
-// the library operation is taken.
+// (rcp/rsqrt.approx.ftz.f64, upper words only: a relative error of 2^-19 at
+// most) with residual e = 1 - x y gives 1/x = y / (1 - e) = y (1 + e + e^2) +
+// O(e^3): 2^-57 relative, then one rounding, in three instructions.  Outside
+// 2^+-1000 the seed would flush and the library operation is taken.  The
+// bounds, the ends of the range and zeros, infinities and NaN are checked
+// against CUDA's operations by tests/test_gpu_fp64.py.
 #pragma once
 
 namespace mm {
@@ -31,13 +33,28 @@ __device__ __forceinline__ double rcp64(double x)
     return __fma_rn(y, __fma_rn(e, e, e), y);
 }
 
-// a / b with the quotient's own residual folded back in
+// |x| in [2^-500, 2^500): a quotient of two such, and its residual, are far
+// from the ends of the range
+__device__ __forceinline__ bool mid_range(double x)
+{
+    return (((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 523u < 1000u;
+}
+
+// a / b with the quotient's own residual folded back in.  Anything else than
+// two numbers of the middle range is the library's quotient (infinities, NaN,
+// a residual that would underflow), but for the frequent zero dividend.
 __device__ __forceinline__ double div64(double a, double b)
 {
-    const double y = rcp64(b), q = __dmul_rn(a, y);
-    const double r = __fma_rn(__fma_rn(-b, q, a), y, q);
-    // a quotient near the range's ends (zero is exact): the library's
-    return seed_range(q) || (__double_as_longlong(q) << 1) == 0 ? r : quot_any(a, b);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double e = __fma_rn(-b, y, 1.0);
+    y = __fma_rn(y, __fma_rn(e, e, e), y);
+    const double q = __dmul_rn(a, y);
+    if (mid_range(b)) {
+        if (mid_range(a)) return __fma_rn(__fma_rn(-b, q, a), y, q);
+        if ((__double_as_longlong(a) << 1) == 0) return q;
+    }
+    return quot_any(a, b);
 }
 
 // 1 / sqrt(x), x > 0: with e = 1 - x y^2, y (1 + e/2 + 3 e^2 / 8)
