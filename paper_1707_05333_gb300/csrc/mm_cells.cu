@@ -69,13 +69,6 @@ struct __align__(16) CellSmem {
 // eight blocks of two warps (eight cells each) an SM; the cells of a warp start in different banks
 static_assert(sizeof(CellSmem) % 32 == 16 && 8 * (8 * sizeof(CellSmem) + 1024) <= 228 * 1024, "shared memory of a cell");
 
-__device__ __forceinline__ float sqrt_fast(float x)
-{
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // Bins of the search shells r = 1 (with the home bin) .. CELL_RINGS in k_clip's order and
 // chunks of 32 of the (2r+1)^3 block: offsets + 8 as x | y << 4 | z << 8, and
 // where each chunk starts.
@@ -144,6 +137,21 @@ __device__ __noinline__ double4_32a vertex_exact(const CellSmem &S, unsigned tri
     solve64(a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, v.x, v.y, v.z);
     v.w = 0.0;
     return v;
+}
+
+// A new vertex and its error bound, k_clip's bits (the gather threshold is
+// formed from them, and the same candidates have to meet in a batch).
+__device__ __forceinline__ float4 cell_vertex(const CellSmem &S, unsigned tri, const double4_32a *__restrict__ sorted,
+                                              const BoxDev *gp)
+{
+    const float4 Pa = S.pf[tri & 31u], Pb = S.pf[(tri >> 5) & 31u], Pc = S.pf[tri >> 10];
+    float x, y, z, er;
+    solve32(Pa, Pb, Pc, plane_length(Pa.w), plane_length(Pb.w), plane_length(Pc.w), x, y, z, er);
+    if (!(er < 1e30f)) {
+        const double4_32a X = vertex_exact(S, tri, sorted, gp);
+        rounded_vertex(X.x, X.y, X.z, x, y, z, er);
+    }
+    return make_float4(x, y, z, er);
 }
 
 // The margin rule of k_clip's plane test on the exact vertex and plane.
@@ -566,7 +574,7 @@ warp_geometry(GeomSmem &S, int lane, int64_t w0, int w, int nt, const BoxDev *gp
     }
 }
 
-// Largest |v|^2 bound of a cell's vertices, (|v| + err)^2 <= |v|^2 + err (2 |v|_1 + err).
+// Largest |v|^2 bound of a cell's vertices (vertex_r2).
 // Formed when candidates are gathered or screened, not at every cut.
 template <int G>
 __device__ __forceinline__ float r2_max(const CellSmem &S, int nt, int gl)
@@ -575,10 +583,9 @@ __device__ __forceinline__ float r2_max(const CellSmem &S, int nt, int gl)
 #pragma unroll 1
     for (int t = gl; t < nt; t += G) {
         const float4 V = S.tf[t];
-        const float s2 = fmaf(V.x, V.x, fmaf(V.y, V.y, V.z * V.z)), l1 = fabsf(V.x) + fabsf(V.y) + fabsf(V.z);
         // (a corner of the starting box has no error; the factors are k_clip's, so
         // that the same candidates are gathered)
-        mr = fmaxf(mr, fmaf(V.w, fmaf(2.0f, l1, V.w), s2) * (V.w == 0.0f ? 1.000001f : 1.00001f));
+        mr = fmaxf(mr, vertex_r2(V.x, V.y, V.z, V.w) * (V.w == 0.0f ? 1.000001f : 1.00001f));
     }
 #pragma unroll
     for (int o = G / 2; o >= 1; o >>= 1) mr = fmaxf(mr, __shfl_xor_sync(FULL, mr, o));
@@ -952,19 +959,8 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
             for (int i = gl; i - gl < maxnew; i += G) {
                 if (go && i < nnew) {
                     const unsigned v = S.tri[i];
-                    float x, y, z, er;
-                    {
-                        const float4 Pa = S.pf[v & 31u], Pb = S.pf[(v >> 5) & 31u], Pc = S.pf[v >> 10];
-                        solve32(Pa, Pb, Pc, sqrt_fast(2.0f * Pa.w), sqrt_fast(2.0f * Pb.w), sqrt_fast(2.0f * Pc.w), x, y, z,
-                                er);
-                    }
-                    if (!(er < 1e30f)) {
-                        const double4_32a X = vertex_exact(S, v, sorted, gp);
-                        x = (float)X.x; y = (float)X.y; z = (float)X.z;
-                        er = 1.2e-7f * (fabsf(x) + fabsf(y) + fabsf(z)) + 1e-38f;
-                    }
                     const int t = i < nrem ? (int)S.hole[i] : nt + i - nrem;
-                    S.tf[t] = make_float4(x, y, z, er);
+                    S.tf[t] = cell_vertex(S, v, sorted, gp);
                     S.vtri[t] = (unsigned short)v;
                 }
             }

@@ -404,15 +404,10 @@ __device__ __forceinline__ void new_vertex(const S_t &S, unsigned nvt, int kp, l
             // its FP32 rounding, whose error is then one rounding per axis
             double X, Y, Z;
             vertex64_call(S, nvt & 255u, (nvt >> 8) & 255u, kp, X, Y, Z);
-            x = (float)X; y = (float)Y; z = (float)Z;
-            er = 1.2e-7f * (fabsf(x) + fabsf(y) + fabsf(z)) + 1e-38f;
+            rounded_vertex(X, Y, Z, x, y, z, er);
         }
         nf = make_float4(x, y, z, er);
-        // an FP32 upper bound of (|v| + er)^2 <= |v|^2 + er (2 |v|_1 + er),
-        // kept as the bit pattern of a positive float
-        const float s2 = fmaf(x, x, fmaf(y, y, z * z));
-        const float l1 = fabsf(x) + fabsf(y) + fabsf(z);
-        nr2 = (long long)__float_as_int(fmaf(er, fmaf(2.0f, l1, er), s2) * 1.00001f);
+        nr2 = (long long)__float_as_int(vertex_r2(x, y, z, er) * 1.00001f);  // the bits of a positive float
     }
 }
 
@@ -508,7 +503,7 @@ __device__ void clip_by(ClipSmem<PREC, CAP> &S, int k, CellState &C, int lane)
         S.pnb[kp] = S.cid[k]; S.psh[kp] = S.csh[k];
         if constexpr (PREC == 1) {
             S.pf[kp] = make_float4(fqx, fqy, fqz, foff);
-            S.pfn[kp] = sqrtf(2.0f * foff);
+            S.pfn[kp] = plane_length(foff);
         }
     }
     __syncwarp();
@@ -787,7 +782,7 @@ clip_cell(ClipSmem<PREC, CAP> &S, const int64_t w, const bool strict, const int 
             const float Lf = gp->Lf[d];
             const float sLf = (lane & 1) ? -Lf : Lf;  // (float)(+-L)
             S.pf[lane] = make_float4(d == 0 ? sLf : 0.0f, d == 1 ? sLf : 0.0f, d == 2 ? sLf : 0.0f, fo);
-            S.pfn[lane] = sqrtf(2.0f * fo);
+            S.pfn[lane] = plane_length(fo);
         }
     } else if (lane < 15) {
         // image offsets s L - p of the three axes (lanes 6..14: axis, s)

@@ -71,12 +71,28 @@ __device__ __forceinline__ long long r2_bits64(double x, double y, double z)
     return __double_as_longlong(__fma_rn(x, x, __fma_rn(y, y, __dmul_rn(z, z))));
 }
 
+// Square root within 2^-23 (the hardware's), for bounds
+__device__ __forceinline__ float sqrt_fast(float x)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// FP32 |q| of a plane with offset o = |q|^2 / 2, for the error bound below (the
+// correctly rounded root costs the grouped clipper, which forms three of them a
+// vertex, 1.5 %: 512 boxes 194.2 -> 197.7 ms)
+__device__ __forceinline__ float plane_length(float o) { return sqrt_fast(2.0f * o); }
+
 // Intersection of planes a, b, c in FP32 with a bound on its distance to the
 // exact intersection.  With P = |q_a||q_b||q_c|, H = P / |det| >= 1 and
 // u = 2^-24, first-order rounding analysis of Cramer's rule (inputs rounded
 // to FP32, cross products, determinant, numerator, scaling) gives
-// |v~ - v| <= u H (5.5 sum|q| + 13 |v|); the bound used is three times that.
+// |v~ - v| <= u H (5.5 sum|q| + 13 |v|); the bound used is three times that,
+// which covers the roundings of the bound itself (plane_length's, H's).
 // Ill-conditioned intersections get an infinite bound (always checked in FP64).
+// la, lb, lc are the planes' |q| (plane_length).  Products that feed a sum are
+// written as such, so that every kernel gets the same bits.
 __device__ __forceinline__ void solve32(const float4 Pa, const float4 Pb, const float4 Pc, float la, float lb, float lc,
                                         float &x, float &y, float &z, float &err)
 {
@@ -88,20 +104,35 @@ __device__ __forceinline__ void solve32(const float4 Pa, const float4 Pb, const 
     const float abx = fmaf(ay, bz, -az * by), aby = fmaf(az, bx, -ax * bz), abz = fmaf(ax, by, -ay * bx);
     const float det = fmaf(ax, bcx, fmaf(ay, bcy, az * bcz));
     const float inv = __frcp_rn(det);
-    x = fmaf(ao, bcx, fmaf(bo, cax, co * abx)) * inv;
-    y = fmaf(ao, bcy, fmaf(bo, cay, co * aby)) * inv;
-    z = fmaf(ao, bcz, fmaf(bo, caz, co * abz)) * inv;
-    // la, lb, lc: |q_k| = sqrt(2 o_k)
+    x = __fmul_rn(fmaf(ao, bcx, fmaf(bo, cax, co * abx)), inv);
+    y = __fmul_rn(fmaf(ao, bcy, fmaf(bo, cay, co * aby)), inv);
+    z = __fmul_rn(fmaf(ao, bcz, fmaf(bo, caz, co * abz)), inv);
     const float H = la * lb * lc * fabsf(inv);  // P / |det| through the reciprocal (the factor 3 covers its ulp)
     const float vn = fabsf(x) + fabsf(y) + fabsf(z);
     const float u = 5.9604645e-8f;
-    err = 3.0f * u * H * (5.5f * (la + lb + lc) + 13.0f * vn);
+    err = __fmul_rn(3.0f * u * H, fmaf(5.5f, la + lb + lc, 13.0f * vn));
     // The analysis assumes no FP32 underflow or overflow: the numerators grow
     // like |q|^4 and the determinant like |q|^3, so planes much nearer than
     // 2^-28 or farther than 2^28 (tiny or huge boxes) are solved exactly.
     const float qlo = fminf(la, fminf(lb, lc)), qhi = fmaxf(la, fmaxf(lb, lc));
     if (!(u * H < 1e-3f) || !(err < 1e30f) || !(qlo >= 3.7252903e-9f) || !(qhi <= 268435456.0f))
         err = __int_as_float(0x7f800000);  // +inf
+}
+// An ill-conditioned intersection is solved in FP64; of its FP32 rounding the
+// error is then one rounding per axis.
+__device__ __forceinline__ void rounded_vertex(double X, double Y, double Z, float &x, float &y, float &z, float &err)
+{
+    x = (float)X;
+    y = (float)Y;
+    z = (float)Z;
+    err = fmaf(1.2e-7f, fabsf(x) + fabsf(y) + fabsf(z), 1e-38f);
+}
+// FP32 bound of (|v| + err)^2 <= |v|^2 + err (2 |v|_1 + err), short of a factor
+// that covers its roundings.
+__device__ __forceinline__ float vertex_r2(float x, float y, float z, float err)
+{
+    const float l1 = fabsf(x) + fabsf(y) + fabsf(z);
+    return fmaf(err, fmaf(2.0f, l1, err), fmaf(x, x, fmaf(y, y, __fmul_rn(z, z))));
 }
 template <class S_t>
 __device__ __forceinline__ void vertex32(const S_t &S, int a, int b, int c, float &x, float &y, float &z,
