@@ -171,37 +171,69 @@ __device__ __forceinline__ unsigned cand_key(float half_d2, unsigned base)
     return min(b > base ? b - base : 0u, 0x7ffffffu) >> 1;
 }
 
-// Candidate order (|q|^2, id, image code) of buffer entries a, b, exactly.
-__device__ __noinline__ bool cand_before(const CellSmem &S, unsigned a, unsigned b,
+// Put the entries of a cell's sorted buffer whose key bits are equal in exact
+// order (|q|^2, id, image code): each lane ranks its entries among those of
+// the same key.  A tied candidate holds |q|^2 / 2 and its id in its plane's
+// place meanwhile.  On exact lattices most entries are tied (runs of 8, 6, 12
+// and 24 on a body-centred one); sorting a run by insertion on one lane, from
+// the generators anew for each comparison, took most of the time there.
+// Tessellation, insertion / rank (warp per cell): body-centred 2 x 16^3 0.51 /
+// 0.33 ms (0.43), 2 x 40^3 4.65 / 2.42 (4.34), cubic 64^3 9.2 / 6.0 (15.1).
+template <int G>
+__device__ __noinline__ void settle_ties(CellSmem &S, int m, unsigned base, int gl,
                                          const double4_32a *__restrict__ sorted, const BoxDev *gp)
 {
-    const unsigned ra = S.cid[a], rb = S.cid[b];
-    const long long da = __double_as_longlong(plane_call(S.off, ra, sorted, gp).w),
-                    db = __double_as_longlong(plane_call(S.off, rb, sorted, gp).w);
-    if (da != db) return da < db;
-    const long long ia = __double_as_longlong(sorted[ra & IDX_MASK].w), ib = __double_as_longlong(sorted[rb & IDX_MASK].w);
-    if (ia != ib) return ia < ib;
-    return (ra >> 27) < (rb >> 27);
-}
-
-// Put entries with equal key bits in exact order (one lane per cell; sorted input).
-__device__ __noinline__ void settle_ties(CellSmem &S, int m, unsigned base, const double4_32a *__restrict__ sorted,
-                                         const BoxDev *gp)
-{
+    unsigned char *const order = reinterpret_cast<unsigned char *>(S.tri);
+    static_assert(sizeof(S.tri) >= CCB, "the new order fits in the new triangles' place");
+    const auto key = [&](int e) { return cand_key(S.cf[S.perm[e]].w, base); };
+    unsigned tied = 0;  // bit i: this lane's entry gl + G i
 #pragma unroll 1
-    for (int k = 1; k < m; ++k) {
-        const unsigned v = S.perm[k];
-        const unsigned kv = cand_key(S.cf[v].w, base);
-        int j = k - 1;
-#pragma unroll 1
-        while (j >= 0) {
-            const unsigned u = S.perm[j];
-            if (cand_key(S.cf[u].w, base) != kv || !cand_before(S, v, u, sorted, gp)) break;
-            S.perm[j + 1] = (unsigned char)u;
-            --j;
-        }
-        S.perm[j + 1] = (unsigned char)v;
+    for (int e = gl, i = 0; e < m; e += G, ++i) {
+        const int v = S.perm[e];
+        const unsigned kv = key(e);
+        order[e] = (unsigned char)v;
+        if (!((e > 0 && key(e - 1) == kv) || (e + 1 < m && key(e + 1) == kv))) continue;
+        tied |= 1u << i;
+        const unsigned ref = S.cid[v];
+        const double o = plane_call(S.off, ref, sorted, gp).w;
+        const int id = (int)__double_as_longlong(sorted[ref & IDX_MASK].w);
+        S.cf[v].x = __int_as_float(__double2loint(o));
+        S.cf[v].y = __int_as_float(__double2hiint(o));
+        S.cf[v].z = __int_as_float(id);
     }
+    __syncwarp();
+    const auto before = [&](int u, int v) {  // buffer entries
+        const float4 U = S.cf[u], V = S.cf[v];
+        const unsigned long long du = (unsigned long long)__float_as_uint(U.y) << 32 | __float_as_uint(U.x),
+                                 dv = (unsigned long long)__float_as_uint(V.y) << 32 | __float_as_uint(V.x);
+        if (du != dv) return du < dv;
+        if (__float_as_int(U.z) != __float_as_int(V.z)) return __float_as_int(U.z) < __float_as_int(V.z);
+        return (S.cid[u] >> 27) < (S.cid[v] >> 27);
+    };
+#pragma unroll 1
+    for (unsigned r = tied; r; r &= r - 1u) {
+        const int e = gl + G * (__ffs((int)r) - 1), v = S.perm[e];
+        const unsigned kv = key(e);
+        int at = e;
+#pragma unroll 1
+        for (int j = e - 1; j >= 0 && key(j) == kv; --j) at -= before(v, S.perm[j]) ? 1 : 0;
+#pragma unroll 1
+        for (int j = e + 1; j < m && key(j) == kv; ++j) at += before(S.perm[j], v) ? 1 : 0;
+        order[at] = (unsigned char)v;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int e = gl, i = 0; e < m; e += G, ++i) {
+        const int v = order[e];
+        if ((tied >> i) & 1u) {  // (its entry is tied too: a run keeps its place)
+            const double4_32a q = plane_call(S.off, S.cid[v], sorted, gp);
+            S.cf[v].x = (float)q.x;
+            S.cf[v].y = (float)q.y;
+            S.cf[v].z = (float)q.z;
+        }
+        S.perm[e] = (unsigned char)v;
+    }
+    __syncwarp();
 }
 
 // Fill the holes a cut left beyond its new vertices from the end of the list
@@ -775,10 +807,7 @@ k_cells(const double4_32a *__restrict__ sorted, const float4 *__restrict__ sorte
             const bool tie = maxm <= 32 ? sort_batch<G, 32 / G>(S, m, kbase, gl) : sort_batch<G, 64 / G>(S, m, kbase, gl);
             const bool gtie = gball(tie) != 0u;
             __syncwarp();
-            if (__any_sync(FULL, gtie)) {
-                if (gtie && gl == 0) settle_ties(S, m, kbase, sorted, gp);
-                __syncwarp();
-            }
+            if (__any_sync(FULL, gtie)) settle_ties<G>(S, gtie ? m : 0, kbase, gl, sorted, gp);
         }
         // Candidates before `fit` are tried one by one; the rest are first
         // screened, a candidate to a lane, against the cell as it is by then: the
