@@ -449,6 +449,12 @@ static mm_status ensure_tess_buffers(mm_ctx *c, int64_t n)
     return MM_OK;
 }
 
+// Whether the grouped clipper takes the cells of a tessellation of n generators.
+static bool grouped_clipper(const mm_ctx *c, int64_t n)
+{
+    return c->cfg.clip_filter && !c->cfg.collect_stats && n >= CELLS_MIN;
+}
+
 // Enqueue the tessellation of the boxes set up last.  fixed: the face arrays
 // already have their capacities and the face count stays on the device.
 static mm_status tess_enqueue(mm_ctx *c, const double *pos, bool fixed)
@@ -487,7 +493,7 @@ static mm_status tess_enqueue(mm_ctx *c, const double *pos, bool fixed)
     // with the face counts written later).  The work counters are those of the
     // warp-per-cell clipper.
     int *list = nullptr;
-    if (prec == 1 && !c->cfg.collect_stats && n >= CELLS_MIN) {
+    if (grouped_clipper(c, n)) {
         list = P<int>(c->emit_cnt);
         launch_cells(P<double4_32a>(c->sorted), P<float4>(c->sortedf), P<int>(c->bin_start), n, boxes, cbox,
                      c->cfg.cand_cap, P<double>(c->vol), P<double>(c->cen), sl, list, &c->st->nlist, s);
@@ -1101,15 +1107,22 @@ mm_status mm_autotune(mm_ctx *c, const double *pos, int64_t n, const double box[
     mm_config best_cfg = keep;
     mm_status r = MM_OK;
     c->timing = 0;
+    // Settings of the warp-per-cell clipper are timed only where it has a share
+    // of the cells: all of them, or a sixteenth on the grouped clipper's list.
+    // Elsewhere their times differ by noise, and the luckiest would stay set
+    // for this context's smaller boxes.
+    r = mm_tessellate(c, pos, n, box, nullptr);
+    const bool share = !grouped_clipper(c, n) || 16 * (int64_t)c->st_host->nlist >= n;
     for (double sc : scale_opt)
         for (int wp : warps_opt)
             for (int cap : cap_opt)
                 for (int so : sort_opt) {
+                if (!share && (wp != warps_opt[0] || so != sort_opt[0])) continue;
                 c->cfg = keep;
                 c->cfg.bin_scale = sc;
-                c->cfg.clip_warps = wp;
+                c->cfg.clip_warps = share ? wp : keep.clip_warps;
                 c->cfg.cand_cap = cap;
-                c->cfg.clip_sort = so;
+                c->cfg.clip_sort = share ? so : keep.clip_sort;
                 double tot = 0.0;
                 for (int k = 0; k < reps + 1 && r == MM_OK; ++k) {
                     cudaEventRecord(e0, c->stream);
