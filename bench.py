@@ -123,11 +123,16 @@ def clocks_stop(proc, path):
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
 # Algorithmic flops per unit of clipping work: a plane test q.v > o
-# (2 FMA + 1 MUL -> 5 flops), a three-plane solve (3 cross products, the
-# determinant, the reciprocal and the scaled numerators -> 51 flops), and a
+# (2 FMA + 1 MUL -> 5 flops), a three-plane solve (two cross-product-like
+# vectors, the determinant, three numerators, the reciprocal and the scaling
+# -> 42 flops), and a
 # face-fan term of the area/centroid sums in the face's own plane (two
 # offsets, a 2-D cross product, three weighted sums -> 12 flops).
-FLOPS_PLANE_TEST, FLOPS_SOLVE, FLOPS_FAN = 5, 51, 12
+FLOPS_PLANE_TEST, FLOPS_SOLVE, FLOPS_FAN = 5, 42, 12
+# Generators from which the filtered clipper is k_cells, with k_clip for the
+# cells it leaves (CELLS_MIN of the library); below, and with the counters on
+# or the direct clipper, k_clip takes every cell.
+GROUPED_MIN = 4096
 # FP32 lanes: 128 per SM per clock, so one FP32 flop costs 1/64 of an FP64
 # flop of issue time on GB300.
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
@@ -169,16 +174,19 @@ def window_direct_counts(ctx, pos, U, box, steps, clip_filter):
 def clip_roofline(direct, filtered, ms, n, clip_filter):
     """FP64 ALU roofline of the clipping kernel: the method's FP64 work
     (clip_method_flops) per launch over the launch's event time, against the
-    FP64 peak.  The FP64-equivalent count of what the filtered kernel itself
-    executes (FP32 tests and solves weighted by the FP64/FP32 peak ratio,
-    plus its FP64 fallbacks, final solves and fans) is kept as an extra key."""
+    FP64 peak.  Where k_clip is the filtered kernel, the FP64-equivalent count
+    of what it executes (FP32 tests and solves weighted by the FP64/FP32 peak
+    ratio, plus its FP64 fallbacks, final solves and fans) is kept as an extra
+    key; the counters of the filtered clipper are k_clip's, so k_cells, which
+    screens its candidates differently, has no such count."""
+    grouped = bool(clip_filter) and n >= GROUPED_MIN
     f_method = clip_method_flops(direct)
     ach = f_method / (ms / 1e3) / 1e12
-    out = {"kernel": "k_cells" if clip_filter else "k_clip", "bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS,
+    out = {"kernel": "k_cells" if grouped else "k_clip", "bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS,
            "unit": "TFLOP/s (FP64)", "frac": ach / FP64_PEAK_TFLOPS, "traffic": None,
            "peak_source": "derived: 152 SMs x 2 FP64 FMA lanes/clk x 2 flops x 2.07 GHz",
            "fp64_flops_per_launch": f_method, "fp64_flops_per_cell": f_method / n, "launch_ms": ms}
-    if clip_filter:
+    if clip_filter and not grouped:
         f32 = FLOPS_PLANE_TEST * direct["fp64_plane_tests"] + FLOPS_SOLVE * direct["fp64_vertex_solves"]
         f64 = (FLOPS_PLANE_TEST * filtered["fp64_plane_tests"] + FLOPS_SOLVE * filtered["fp64_vertex_solves"] +
                FLOPS_FAN * filtered["fp64_fan_terms"])
@@ -190,13 +198,14 @@ def clip_roofline(direct, filtered, ms, n, clip_filter):
     return out
 
 
-# DRAM traffic of the clipper per cell, from an ncu capture of one k_cells launch
-# on the 128^3 shear layer (dram__bytes_read.sum + dram__bytes_write.sum = 452,787,968
-# + 1,435,980,800 bytes over 2,097,152 cells); it scales with the cells of the launch.
+# DRAM traffic of the grouped clipper per cell, from an ncu capture of one k_cells
+# launch on the 128^3 shear layer; it scales with the cells of the launch.
 # Valid only for the clipper sources it was taken on: the digest of the clipping
-# kernels' sources must match, else the figure is withheld.
-CLIP_TRAFFIC = {"sources": ("csrc/mm_cells.cu", "csrc/mm_clip.cu", "csrc/mm_clip.cuh", "csrc/mm_internal.cuh"),
-                "sha256_16": "317f07aec105e5f7", "bytes_per_cell": 1888768768 / 2097152, "cells_captured": 2097152}
+# kernels' sources must match, else the figure is withheld.  None: not captured
+# on the present sources.
+CLIP_TRAFFIC = {"sources": ("csrc/mm_cells.cu", "csrc/mm_clip.cu", "csrc/mm_clip.cuh", "csrc/mm_fp64.cuh",
+                            "csrc/mm_internal.cuh"),
+                "sha256_16": None, "bytes_per_cell": None, "cells_captured": 2097152}
 
 
 def clip_sources_digest():
@@ -209,10 +218,10 @@ def clip_sources_digest():
 
 
 def clip_traffic(n, clip_filter):
-    """DRAM bytes of the clipping launches on n cells, scaled from the 128^3
+    """DRAM bytes of one k_cells launch on n cells, scaled from the 128^3
     capture by cell count; None when the capture does not cover the current
-    clipper source or clipper variant."""
-    if not clip_filter or CLIP_TRAFFIC["bytes_per_cell"] is None:
+    clipper source or k_cells does not run."""
+    if not clip_filter or n < GROUPED_MIN or CLIP_TRAFFIC["bytes_per_cell"] is None:
         return None
     if clip_sources_digest() != CLIP_TRAFFIC["sha256_16"]:
         return None
@@ -826,7 +835,7 @@ def run_ours(args, world, rank, local):
         roofline = clip_roofline(tdirect, tstats, dom_ms, n, args.clip_filter)
         roofline["traffic"] = clip_traffic(n, args.clip_filter)
         if roofline["traffic"] is not None:
-            roofline["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the clipping launches "
+            roofline["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_cells launch "
                                           "at 128^3, scaled by cells")
     else:
         byts = algorithmic_bytes(dom, n, nf)
