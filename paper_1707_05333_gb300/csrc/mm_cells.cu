@@ -32,6 +32,8 @@
 // new vertices in a cut, CELL_RINGS search rings), holds a coincident
 // generator or has an inconsistent cut goes to a list that the warp-per-cell
 // clipper works through next, so nothing is refused here.
+#include <cstddef>
+
 #include "mm_clip.cuh"
 
 namespace mm {
@@ -367,6 +369,7 @@ struct __align__(16) GeomSmem {
     unsigned char bad[GC];
 };
 static_assert(sizeof(GeomSmem) <= GC * sizeof(CellSmem), "it takes the place of the clipped cells");
+static_assert(offsetof(GeomSmem, nxt) % 16 == 0 && CPM % 16 == 0, "edge rows are read 16 bytes at a time");
 
 __device__ __forceinline__ int plane_of(const GeomSmem &S, int c, unsigned slot)
 {
