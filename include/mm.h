@@ -71,14 +71,17 @@ typedef struct {
     int regularize;   /* 1: add the roundness correction to w (Sec. 4.2)                    */
     int precision;    /* 0: FP64 hydro; 1: mixed (FP32 gradients, half step and fluxes,     */
                       /*    FP64 update); the mesh is FP64-exact either way (clip_filter)   */
-    int collect_stats;/* 1: the clipper records the counters read by mm_tess_stats          */
+    int collect_stats;/* 1: record the counters read by mm_tess_stats; every cell then takes */
+                      /*    the warp-per-cell clipper, whose counters they are (same mesh)   */
     int riemann;      /* 0 HLLC (the paper's default), 1 HLL (Sec. 4)                        */
     int clip_warps;   /* cells (warps) per block of the warp-per-cell clipper, 1..8 (tunable; */
                       /*    2); from 4096 generators on it takes only the unusual cells      */
     int cand_cap;     /* candidates per sorted batch of the clipper, 32..64 (tunable)        */
     int clip_filter;  /* 1: clip with FP32 vertices, an error-bounded FP32 plane test and    */
-                      /*    an exact FP64 test near ties, then FP64 vertices (same mesh, bit */
-                      /*    for bit); 0: solve and test every vertex in FP64 as it appears  */
+                      /*    an exact FP64 test near ties, then FP64 vertices; 0: solve and   */
+                      /*    test every vertex in FP64 as it appears.  The cells are the same; */
+                      /*    in rare ones the faces come in another order (the limits up to   */
+                      /*    which candidates are gathered differ by rounding)                */
     double bin_scale; /* neighbour-search bin edge in mean generator spacings (tunable)       */
     double mach_th;   /* energy/entropy switch: a cell whose largest face shock Mach number   */
                       /*    is below mach_th takes its energy from its entropy (Sec. 4.3);   */

@@ -11,10 +11,12 @@
 // What bounds it and what it measured (GB300, jittered 64^3 lattice and
 // 200003 random generators, ncu durations; k_clip took 5.89 and 8.89 ms):
 // 2.6 and 4.2 ms, of dependent latencies with 15 warps an SM (3.4 KB of
-// shared memory a cell, 128 registers): 1.6 instructions a cycle, 5220 a cell
-// against k_clip's 14200, and the FP64 pipe 52 % busy with 107 instructions a
-// cell against 236.  (18 warps an SM at 96 registers gained nothing: the
-// misses of the instruction cache doubled.)
+// shared memory a cell, 128 registers): 1.6 instructions a cycle, 4920 a cell
+// against k_clip's 14200, and the FP64 pipe 55 % busy with 108 instructions a
+// cell against 236.  Random cells take 11600 instructions at 1.8 a cycle, with
+// 19 active lanes for the lattice's 24: cells of unlike length share a warp.
+// (18 warps an SM at 96 registers gained nothing: the misses of the
+// instruction cache doubled.)
 //  * Loops are kept rolled: unrolled, the body outgrew the instruction cache
 //    and half of the cycles went to fetching it (5.3 and 13.0 ms).
 //  * Screening candidates a lane each after the first SCREEN instead of trying

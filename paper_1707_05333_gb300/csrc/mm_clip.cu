@@ -1,5 +1,8 @@
 // mm_clip.cu -- Voronoi cells by half-space clipping, one warp per cell (Sec. 3).
 //
+// It takes every cell of small sets, of the direct FP64 variant and of counted
+// runs; otherwise the cells that the grouped clipper (mm_cells.cu) leaves.
+//
 // The paper builds each cell by starting from a large box around the
 // generator p and cutting it with the bisector plane of every neighbour n,
 // nearest first, until |n - p| exceeds twice the distance to the farthest
@@ -47,8 +50,8 @@ constexpr int CBATCH = 64;  // candidate buffer; flushed (sorted + clipped) when
 
 // Per-cell capacities of one instance of the clipper: planes, vertices, new
 // vertices per cut, faces written, search rings and edge-table slots.  The
-// main instance runs every cell; the large one re-clips the cells that
-// overflowed the main one's lists.
+// main instance runs every cell of a launch; the large one re-clips the cells
+// that overflowed the main one's lists.
 template <int PM_, int TM_, int NS_, int MF_, int MR_, int ETAB_, bool BIG_>
 struct Caps {
     static constexpr int PM = PM_, TM = TM_, NS = NS_, MF = MF_, MR = MR_, ETAB = ETAB_;
@@ -951,8 +954,10 @@ clip_cell(ClipSmem<PREC, CAP> &S, const int64_t w, const bool strict, const int 
     // triangle (x, y, z) maps to that triangle and z, so the next vertex
     // around a face is one lookup.  Keys are unique in a closed
     // triangulation; the load stays below 3/4 (else the walk scans instead).
-    // A face starts at the triangle of its edge to the lowest plane slot (an
-    // order of the triangles that no schedule can change).
+    // With the table a face starts at the triangle of its edge to the lowest
+    // plane slot (an order of the triangles that no schedule can change, and the
+    // grouped clipper's); without, in cells of more than 64 vertices, which that
+    // one never finishes, at the first triangle of the list.
     constexpr int ETAB = CAP::ETAB, PB = CAP::PB, TB = CAP::TB;
     const bool use_tab = !C.err && 3 * C.nt <= (3 * ETAB) / 4;
     unsigned *etab = S.u.f.etab;

@@ -434,10 +434,11 @@ void launch_gradient(const MeshDev &m, const HydroCfg &c, const double *W, const
 // ---------------------------------------------------------------------------
 using FaceState = FaceStateT<double>;
 
-// Bound by the FP64 pipe (90 % busy at 234 instructions a face): the count is
+// Bound by the FP64 pipe (89 % busy at 200 instructions a face): the count is
 // the cost.  Reciprocals of mm_fp64.cuh, two operations a momentum component
 // (hllc_t), floors compared as integers and no offsets added to faces inside
-// the box: 54.2 -> 47.5 ms for the 133 million faces of the 256^3 shear layer.
+// the box: 54.2 -> 47.5 ms for the 133 million faces of the 256^3 shear layer,
+// 234 -> 200 instructions with the short square roots.
 // With NG = 6 the flux rows 5, 6 and 7 hold the entropy flux A F_(rho A), the
 // face's shock Mach number and its swept-volume rate A (w_f . n).
 template <int NG>

@@ -28,9 +28,14 @@ constexpr int NUM_SMS = 152;       // GB300
 constexpr int CLIP_MAX_WARPS = 8;  // warps (cells) per block of the clipper, tunable at run time
 // Cells from which the grouped clipper (mm_cells.cu) runs.  Below, the chip is
 // not full and a warp per cell finishes sooner.  Tessellation, warp per cell
-// against grouped: 2000 random generators 0.35 / 0.41 ms, 4100 0.44 / 0.45,
-// 8000 0.65 / 0.48, 200003 9.6 / 4.9; jittered lattices 12^3 0.20 / 0.23,
-// 16^3 0.27 / 0.24, 20^3 0.38 / 0.27, 64^3 6.3 / 3.2.
+// against grouped: 2000 random generators 0.35 / 0.41 ms, 4500 0.46 / 0.47,
+// 5000 0.47 / 0.43, 6000 0.52 / 0.45, 8000 0.61 / 0.45, 200003 9.6 / 5.1;
+// jittered lattices 12^3 0.20 / 0.23, 16^3 0.28 / 0.24, 20^3 0.38 / 0.27, 64^3
+// 6.3 / 3.1; exact cubic 16^3 0.38 / 0.28.  Where a few cells take longest and
+// overflow the lists of both clippers, their times add up: a third of the
+// generators in a plane, 4500 1.06 / 1.34, 9000 1.69 / 1.80, 100000 8.7 / 5.7;
+// with half of the generators in crowded bins (clustered) the grouped clipper
+// gains nothing and costs 1 % (200000) or less.
 constexpr int64_t CELLS_MIN = 4096;
 // Overflow rows reserved when the count of retried cells is not known in
 // advance (graph mode); mm_tessellate sizes them to the count it reads.

@@ -113,3 +113,17 @@ def test_batch_of_the_grouped_clipper_equals_boxes_alone(precision, integrator):
                 assert float(dt[b].item()) == float(d1.item()), (b, step)
         one.close()
         ref.close()
+
+
+@pytest.mark.parametrize("value", [np.nan, -1e-9, 1.0, 1.5])
+def test_generators_outside_the_box_are_refused(ctx, value):
+    """One generator that is not in the box, and a whole warp of them: the
+    call is refused and the context stays usable."""
+    from paper_1707_05333_gb300 import binding
+    c, torch = ctx
+    for bad in ([17], list(range(40, 72))):
+        pos = WL.random_points(5003, seed=52)
+        pos[bad, 1] = value
+        with pytest.raises(binding.MMError, match="outside"):
+            H.gpu_tessellate(c, torch, pos, np.ones(3))
+    assert abs(H.gpu_tessellate(c, torch, WL.random_points(5003, seed=52), np.ones(3))[2]["cell_volume"].sum() - 1.0) < 1e-12
