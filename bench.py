@@ -199,13 +199,14 @@ def clip_roofline(direct, filtered, ms, n, clip_filter):
 
 
 # DRAM traffic of the grouped clipper per cell, from an ncu capture of one k_cells
-# launch on the 128^3 shear layer; it scales with the cells of the launch.
-# Valid only for the clipper sources it was taken on: the digest of the clipping
-# kernels' sources must match, else the figure is withheld.  None: not captured
-# on the present sources.
+# launch on the 128^3 shear layer (dram__bytes_read.sum + dram__bytes_write.sum =
+# 452,394,496 + 1,435,896,064 bytes over 2,097,152 cells); it scales with the cells
+# of the launch.  Valid only for the clipper sources it was taken on: the digest of
+# the clipping kernels' sources must match, else the figure is withheld (None: not
+# captured on the present sources).
 CLIP_TRAFFIC = {"sources": ("csrc/mm_cells.cu", "csrc/mm_clip.cu", "csrc/mm_clip.cuh", "csrc/mm_fp64.cuh",
                             "csrc/mm_internal.cuh"),
-                "sha256_16": None, "bytes_per_cell": None, "cells_captured": 2097152}
+                "sha256_16": "79982821a75a4a39", "bytes_per_cell": 1888290560 / 2097152, "cells_captured": 2097152}
 
 
 def clip_sources_digest():
